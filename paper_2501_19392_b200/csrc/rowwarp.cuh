@@ -11,12 +11,11 @@
 //                   element index bits 0, 1, 2, 8, 9 select a register  -> five stages in registers
 //   transposition   through a 4 KB shared-memory buffer of the warp: within each half-warp the
 //                   pair index k (bits 1, 2, 8, 9) trades places with the lane index (bits 3..6)
-//   bit 7           separates the half-warps in both layouts: a lane reads the other half's item of the
-//                   transposition beside its own
+//   bit 7           separates the half-warps in both layouts                -> one shuffle stage
 //   search layout   lane L', pair m holds elements with bits 3..6 = m, bits (1, 2, 8, 9) = L' % 16,
 //                   bit 7 = L' / 16                                        -> four stages in registers
 // The two values that share a code (2j, 2j+1) stay in one register pair throughout.  Compared with
-// a row spread over four warps (codec.cuh) this removes the five shuffle stages and all
+// a row spread over four warps (codec.cuh) this removes four of the five shuffle stages and all
 // cross-warp barriers: the row work is bound by the SM's load/store and shuffle pipe, which the
 // tensor-core GEMM beside it also needs for its operand reads.
 //
@@ -76,40 +75,54 @@ __device__ __forceinline__ void wr_stage_regs(f32x2_t (&vp)[16]) {
   }
 }
 
-// Trades the pair index for the low four lane bits inside each half-warp (afterwards pair m of lane l holds what pair l
-// of lane m held) and adds the butterfly over element index bit 7, which separates the half-warps before and after.
-// Rows are 17 items apart, so the 16 lanes of a half-warp touch 16 different 8-byte columns both when they write (row k)
-// and when they read (row = lane), and every access is a fixed offset from one address of the lane: an exclusive-or
-// swizzle needed an address of its own per access, and the butterfly 32 shuffles where the second read takes 16.
-// The same call converts in both directions.
-__device__ __forceinline__ void wr_transpose_halves(f32x2_t (&vp)[16], unsigned long long* xbuf, int lane) {
+// Butterfly over element index bit 7, which separates the half-warps in both layouts.
+__device__ __forceinline__ void wr_stage_halves(f32x2_t (&vp)[16], int lane) {
+  const float sg = (lane & 16) ? -1.0f : 1.0f;
+  const f32x2_t sg2 = pack2(sg, sg);
+#pragma unroll
+  for (int m = 0; m < 16; ++m) {
+    float a, b;
+    unpack2(vp[m], a, b);
+    const float oa = __shfl_xor_sync(0xffffffffu, a, 16), ob = __shfl_xor_sync(0xffffffffu, b, 16);
+    vp[m] = fma2(sg2, vp[m], pack2(oa, ob));   // lower half: v + o; upper half: o - v
+  }
+}
+
+// Trades the pair index for the low four lane bits inside each half-warp: afterwards pair m of lane l holds what pair l
+// of lane m held.  Rows are 17 items apart, so the 16 lanes of a half-warp touch 16 different 8-byte columns both when
+// they write (row k) and when they read (row = lane), and every access is a fixed offset from one address of the
+// lane: an exclusive-or swizzle needed an address of its own per access.  The same call converts in both directions.
+__device__ __forceinline__ void wr_transpose(f32x2_t (&vp)[16], unsigned long long* xbuf, int lane) {
   const int l = lane & 15, h = lane >> 4;
   unsigned long long* put = xbuf + h * (16 * kWrPitch) + l;
   const unsigned long long* own = xbuf + h * (16 * kWrPitch) + l * kWrPitch;
-  const unsigned long long* oth = xbuf + (h ^ 1) * (16 * kWrPitch) + l * kWrPitch;
-  const float sg = h ? -1.0f : 1.0f;
-  const f32x2_t sg2 = pack2(sg, sg);
 #pragma unroll
   for (int k = 0; k < 16; ++k) put[k * kWrPitch] = vp[k];
   __syncwarp();
 #pragma unroll
-  for (int m = 0; m < 16; ++m) vp[m] = fma2(sg2, own[m], oth[m]);   // lower half: v + o; upper half: o - v
+  for (int m = 0; m < 16; ++m) vp[m] = own[m];
   __syncwarp();
 }
 
-// H_1024 (unnormalised) from the load layout to the search layout.
+// H_1024 (unnormalised) from the load layout to the search layout.  The order of the stages is part of the result: fp32
+// sums in another order move a reconstruction in a thousand by a unit in the last place and, through it, codes of the
+// tensors predicted from it, so that an encoder would no longer write, and a decoder no longer read, what builds with
+// this order do.  (Bit 7 beside the transposition instead, where the butterfly's partner is a second read of the
+// buffer: no faster in the decoder, 131072 tokens 925 against 912 us, and the encoder 397 against 399 us at 32768.)
 __device__ __forceinline__ void wr_rotate_forward(f32x2_t (&vp)[16], unsigned long long* xbuf, int lane) {
   wr_stage_pair(vp);
   wr_stage_regs(vp);
-  wr_transpose_halves(vp, xbuf, lane);
+  wr_transpose(vp, xbuf, lane);
   wr_stage_regs(vp);
+  wr_stage_halves(vp, lane);
 }
 
 // H_1024 (unnormalised) from the search layout back to the load layout.  Encode and decode both
 // reconstruct through this one routine, so their results agree bit for bit.
 __device__ __forceinline__ void wr_rotate_back(f32x2_t (&wp)[16], unsigned long long* xbuf, int lane) {
+  wr_stage_halves(wp, lane);
   wr_stage_regs(wp);
-  wr_transpose_halves(wp, xbuf, lane);
+  wr_transpose(wp, xbuf, lane);
   wr_stage_regs(wp);
   wr_stage_pair(wp);
 }
@@ -154,27 +167,31 @@ __device__ __forceinline__ void wr_finish_row(const WarpRowCtx& rc, f32x2_t (&wp
                                               typename RowArg<Pred>::type pred_row, const f32x2_t (&pr)[16],
                                               typename RowArg<Hat>::type hat_row) {
   const int lane = rc.lane;
-  auto signed_c = [&](int k) {       // the pair's signs on the scale, so that scale, sign and prediction are one FMA
-    const float a = __uint_as_float(__float_as_uint(c) ^ ((rc.signs << (31 - 2 * k)) & 0x80000000u));
-    const float b = __uint_as_float(__float_as_uint(c) ^ ((rc.signs << (30 - 2 * k)) & 0x80000000u));
-    return pack2(a, b);
+  // the scaled value is rounded before the prediction is added (like the order of the rotation's stages, part of the
+  // result); the product with the sign is exact, so the FMA is that addition
+  const f32x2_t c2 = pack2(c, c);
+  auto sign = [&](int k) {       // (+-1, +-1): the signs of pair k
+    return pack2(__uint_as_float(((rc.signs << (31 - 2 * k)) & 0x80000000u) | 0x3f800000u),
+                 __uint_as_float(((rc.signs << (30 - 2 * k)) & 0x80000000u) | 0x3f800000u));
   };
 #pragma unroll
   for (int ch = 0; ch < 4; ++ch) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) wp[4 * ch + i] = mul2(wp[4 * ch + i], c2);
     if (pred_row != nullptr) {
       if constexpr (kEarly) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) wp[4 * ch + i] = fma2(wp[4 * ch + i], signed_c(4 * ch + i), pr[4 * ch + i]);
+        for (int i = 0; i < 4; ++i) wp[4 * ch + i] = fma2(wp[4 * ch + i], sign(4 * ch + i), pr[4 * ch + i]);
       } else {
         f32x2_t p[4];
         wr_load_pred8(pred_row + (ch * 256 + lane * 8), p);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) wp[4 * ch + i] = fma2(wp[4 * ch + i], signed_c(4 * ch + i), p[i]);
+        for (int i = 0; i < 4; ++i) wp[4 * ch + i] = fma2(wp[4 * ch + i], sign(4 * ch + i), p[i]);
       }
     } else {
       // adding the zero prediction turns a -0 (a zero value whose sign was flipped) into +0
 #pragma unroll
-      for (int i = 0; i < 4; ++i) wp[4 * ch + i] = fma2(wp[4 * ch + i], signed_c(4 * ch + i), pack2(0.0f, 0.0f));
+      for (int i = 0; i < 4; ++i) wp[4 * ch + i] = fma2(wp[4 * ch + i], sign(4 * ch + i), pack2(0.0f, 0.0f));
     }
     const uint4 out = make_uint4(store16x2p<kBf16>(wp[4 * ch + 0]), store16x2p<kBf16>(wp[4 * ch + 1]),
                                  store16x2p<kBf16>(wp[4 * ch + 2]), store16x2p<kBf16>(wp[4 * ch + 3]));

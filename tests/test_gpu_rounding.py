@@ -1,0 +1,89 @@
+"""The row kernels' results bit for bit, from the order in which they round: the rotation's butterflies in single precision stage
+by stage, the normalisation, the search and the reconstruction, restated here with one torch operation per rounding.
+
+A packed cache outlives the build that wrote it, and a chain of layers passes every moved last bit on to codes of the layers
+that follow, so the order is part of what the library promises and not only the accuracy, which the oracle
+tests check.  The prediction is the library's own (aquakv_predict)."""
+import pytest
+import torch
+
+from paper_2501_19392_b200 import synth
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+T = 300
+
+
+def make(d, h, g, dtype, grid=None, levels=0):
+    from paper_2501_19392_b200 import api
+    return api.Codec(d, h, g, grid, dtype, synth.hadamard_signs(d, 11), synth.hadamard_signs(d, 12), levels=levels)
+
+
+def signs(d, role):
+    return torch.from_numpy(synth.hadamard_signs(d, 11 + role)).to(DEV, torch.float32)
+
+
+def butterflies(x, bits):
+    """Unnormalised Hadamard butterflies over the given index bits, in that order, each rounded to fp32."""
+    for b in bits:
+        n, d = x.shape
+        v = x.view(n, d >> (b + 1), 2, 1 << b)
+        x = torch.stack([v[:, :, 0] + v[:, :, 1], v[:, :, 0] - v[:, :, 1]], dim=2).reshape(n, d)
+    return x
+
+
+def fma(a, b, c):
+    """One rounding to fp32: the product of two fp32 values is exact in double (and so, but for one case in 2^29, the sum)."""
+    return (a.double() * b.double() + c.double()).float()
+
+
+def unpack(codes, bits):
+    b = (codes.to(torch.int32)[:, :, None] >> torch.arange(8, device=DEV)) & 1
+    return (b.view(codes.shape[0], -1, bits) << torch.arange(bits, device=DEV)).sum(-1)
+
+
+def rows(codec, d, dtype, seed):
+    shape = (T, d)
+    X = synth.random_16bit(shape, dtype, seed, device=DEV)
+    prev = synth.random_16bit(shape, dtype, seed + 1, device=DEV)
+    W = (synth.random_16bit((d, d), dtype, seed + 2, device=DEV).float() / d ** 0.5).to(X.dtype)
+    P = codec.predict(prev, None, W)
+    return X, prev, W, P
+
+
+def both_ways(codec, X, prev, W, role):
+    codes, scales, hat = codec.encode_phase(role, X, prev, None, W)
+    assert torch.equal(codec.decode_phase(role, codes, scales, prev, None, W), hat)
+    return codes, scales, hat
+
+
+@pytest.mark.parametrize("n,dtype", [(16, synth.BF16), (64, synth.F16), (256, synth.F16)])
+def test_rows_of_one_warp(n, dtype):
+    d = 1024
+    grid = synth.lloyd_grid(n, seed=7, n_samples=1 << 14, iters=20)
+    codec = make(d, d, d, dtype, grid)
+    for role in (0, 1):
+        X, prev, W, P = rows(codec, d, dtype, 5 + 10 * role)
+        codes, scales, hat = both_ways(codec, X, prev, W, role)
+        sg, s = signs(d, role), scales.float()
+        y = butterflies((X.float() - P) * sg, (0, 1, 2, 8, 9, 3, 4, 5, 6, 7)) * ((1.0 / s) * (1.0 / 32.0))
+        g = torch.from_numpy(grid).to(DEV)
+        dx = y.view(T, -1, 2)[:, :, None, :] - g
+        sq = dx * dx
+        q = (sq[..., 0] + sq[..., 1]).argmin(-1)
+        assert torch.equal(unpack(codes, n.bit_length() - 1), q)
+        x = butterflies(g[q].reshape(T, d), (7, 3, 4, 5, 6, 1, 2, 8, 9, 0)) * (s * (1.0 / 32.0))
+        assert torch.equal(hat, (P + x * sg).to(hat.dtype))
+
+
+def test_the_layer_kernel_rounds_like_the_row_kernels():
+    """Keys of the fused encode and decode (whose prediction stays inside the kernel) equal the phase calls' bit for bit."""
+    d, dtype = 1024, synth.BF16
+    codec = make(d, d, d, dtype, synth.lloyd_grid(16, seed=7, n_samples=1 << 14, iters=20))
+    X, prev, W, _ = rows(codec, d, dtype, 40)
+    Wv = torch.cat([W, W], dim=1).contiguous()
+    codes, scales, hat = both_ways(codec, X, prev, W, 0)
+    out = codec.encode(X, X, prev, prev, W, Wv)
+    assert torch.equal(out[0], codes) and torch.equal(out[1], scales) and torch.equal(out[4], hat)
+    Kh, Vh = codec.decode(*out[:4], prev, prev, W, Wv)
+    assert torch.equal(Kh, hat) and torch.equal(Vh, out[5])
