@@ -253,7 +253,7 @@ grid4_encode_rows_kernel(const Grid4Args ga) {
 #pragma unroll
       for (int c = 0; c < NCH; ++c) ss[c] += __shfl_xor_sync(0xffffffffu, ss[c], off);
     }
-    float f[NCH];                          // scale / sqrt(h)
+    float f[NCH];                          // scale
 #pragma unroll
     for (int c0 = 0; c0 < NCH; ++c0) {
       float sum = 0.0f;                    // a group of several chunks: the sum over its chunks
@@ -262,7 +262,7 @@ grid4_encode_rows_kernel(const Grid4Args ga) {
         if ((c & ~(chunks_per_group - 1)) == (c0 & ~(chunks_per_group - 1))) sum += ss[c];
       const __half s16 = __float2half_rn(fminf(sqrtf(sum * inv_g), 65504.0f));
       const float sf = __half2float(s16);
-      f[c0] = sf * rs;
+      f[c0] = sf;
       if ((lane & (lanes_per_group - 1)) == 0 && (c0 & (chunks_per_group - 1)) == 0)
         a.scales[t * n_groups + ((256 * c0 + 8 * lane) >> a.log_g)] = __half_as_ushort(s16);
       const float inv = sf > 0.0f ? __fdiv_rn(1.0f, sf) : 0.0f;
@@ -302,7 +302,7 @@ grid4_encode_rows_kernel(const Grid4Args ga) {
     if (a.hat != nullptr) {
       f32x2_t pred[NCH][4];
       row_load_pred<NCH>(a, t, lane, pred);
-      row_rotate_back<kBf16, NCH>(a, t, lane, ga.log_h, sbits, v, f, pred);
+      row_rotate_back<kBf16, NCH>(a, t, lane, ga.log_h, sbits, rs, v, f, pred);
     }
   }
 }
@@ -327,7 +327,7 @@ grid4_decode_rows_kernel(const Grid4Args ga) {
 #pragma unroll
     for (int c = 0; c < NCH; ++c) {
       const uint32_t two = *reinterpret_cast<const uint16_t*>(a.codes + t * (long long)(a.d / 4) + 64 * c + 2 * lane);
-      f[c] = __half2float(__ushort_as_half(a.scales[t * n_groups + ((256 * c + 8 * lane) >> a.log_g)])) * rs;
+      f[c] = __half2float(__ushort_as_half(a.scales[t * n_groups + ((256 * c + 8 * lane) >> a.log_g)]));
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
         const ulonglong2 g = lds128(grid + ((two >> (8 * u)) & 0xffu) * 16u);
@@ -335,7 +335,7 @@ grid4_decode_rows_kernel(const Grid4Args ga) {
         y[c][2 * u + 1] = g.y;
       }
     }
-    row_rotate_back<kBf16, NCH>(a, t, lane, ga.log_h, sbits, y, f, pred);
+    row_rotate_back<kBf16, NCH>(a, t, lane, ga.log_h, sbits, rs, y, f, pred);
   }
 }
 

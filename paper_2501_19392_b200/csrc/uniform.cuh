@@ -188,15 +188,18 @@ __device__ __forceinline__ void row_store_pair4(uint16_t* dst, const f32x2_t (&h
                                                    store16x2p<kBf16>(h[3])));
 }
 
-// hat = round16(pred + f[c] * signs . H(y)) for the row's values y before the inverse rotation.
+// hat = round16(pred + f[c] * signs . (rs * H(y))) for the row's values y before the inverse rotation.  rs = 1 / sqrt(h)
+// is a rounding of its own, after the rotation in both directions: on the signs before it, which saves a multiplication,
+// it moves last bits wherever it is no power of two (h = 128, 512), and with them codes.
 template <bool kBf16, int NCH>
-__device__ __forceinline__ void row_rotate_back(const UniformArgs& a, long long t, int lane, int log_h, uint32_t sbits,
+__device__ __forceinline__ void row_rotate_back(const UniformArgs& a, long long t, int lane, int log_h, uint32_t sbits, float rs,
                                                 f32x2_t (&y)[NCH][4], const float (&f)[NCH], const f32x2_t (&pred)[NCH][4]) {
   row_hadamard<NCH>(y, log_h, lane);
+  const f32x2_t rs2 = pack2(rs, rs);
 #pragma unroll
   for (int c = 0; c < NCH; ++c) {
 #pragma unroll
-    for (int k = 0; k < 4; ++k) y[c][k] = fma2(y[c][k], row_signed(f[c], sbits, c, k), pred[c][k]);
+    for (int k = 0; k < 4; ++k) y[c][k] = fma2(mul2(y[c][k], rs2), row_signed(f[c], sbits, c, k), pred[c][k]);
     row_store_pair4<kBf16>(a.hat + t * a.ldHat + 256 * c + 8 * lane, y[c]);
   }
 }
@@ -224,8 +227,13 @@ uniform_encode_rows_kernel(const UniformRotArgs ra) {
 #pragma unroll
       for (int c = 0; c < NCH; ++c)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) v[c][k] = mul2(v[c][k], row_signed(rs, sbits, c, k));
+        for (int k = 0; k < 4; ++k) v[c][k] = mul2(v[c][k], row_signed(1.0f, sbits, c, k));
       row_hadamard<NCH>(v, ra.log_h, lane);
+      const f32x2_t rs2 = pack2(rs, rs);
+#pragma unroll
+      for (int c = 0; c < NCH; ++c)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[c][k] = mul2(v[c][k], rs2);
     }
     // group absmax
     float m[NCH];
@@ -273,8 +281,8 @@ uniform_encode_rows_kernel(const UniformRotArgs ra) {
     if constexpr (kRot) {
       float f[NCH];
 #pragma unroll
-      for (int c = 0; c < NCH; ++c) f[c] = rs;
-      if (a.hat != nullptr) row_rotate_back<kBf16, NCH>(a, t, lane, ra.log_h, sbits, v, f, pred);
+      for (int c = 0; c < NCH; ++c) f[c] = 1.0f;
+      if (a.hat != nullptr) row_rotate_back<kBf16, NCH>(a, t, lane, ra.log_h, sbits, rs, v, f, pred);
     }
   }
 }
@@ -318,8 +326,8 @@ uniform_decode_rows_kernel(const UniformRotArgs ra) {
     if constexpr (kRot) {
       float f[NCH];
 #pragma unroll
-      for (int c = 0; c < NCH; ++c) f[c] = rs;
-      row_rotate_back<kBf16, NCH>(a, t, lane, ra.log_h, sbits, y, f, pred);
+      for (int c = 0; c < NCH; ++c) f[c] = 1.0f;
+      row_rotate_back<kBf16, NCH>(a, t, lane, ra.log_h, sbits, rs, y, f, pred);
     }
   }
 }

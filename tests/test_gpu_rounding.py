@@ -87,3 +87,34 @@ def test_the_layer_kernel_rounds_like_the_row_kernels():
     assert torch.equal(out[0], codes) and torch.equal(out[1], scales) and torch.equal(out[4], hat)
     Kh, Vh = codec.decode(*out[:4], prev, prev, W, Wv)
     assert torch.equal(Kh, hat) and torch.equal(Vh, out[5])
+
+
+def rsqrt(h):
+    return torch.rsqrt(torch.tensor(float(h), device=DEV))
+
+
+@pytest.mark.parametrize("d,h,g,levels,dtype", [(512, 512, 128, 8, synth.F16), (1024, 128, 1024, 16, synth.BF16), (256, 64, 32, 4, synth.F16)])
+def test_uniform_levels_after_a_rotation(d, h, g, levels, dtype):
+    codec = make(d, h, g, dtype, None, levels)
+    order, half = range(h.bit_length() - 1), levels // 2
+    for role in (0, 1):
+        X, prev, W, P = rows(codec, d, dtype, 60 + 10 * role)
+        codes, scales, hat = both_ways(codec, X, prev, W, role)
+        sg, rs = signs(d, role), rsqrt(h)
+        v = butterflies((X.float() - P) * sg, order) * rs
+        assert torch.equal((v.view(T, d // g, g).abs().amax(-1) * (1.0 / half)).half(), scales)
+        sf = scales.float().repeat_interleave(g, dim=1)
+        level = torch.clamp(torch.ceil(v.double() / sf.double() - 0.5), -half, half - 1).float()
+        assert torch.equal(unpack(codes, levels.bit_length() - 1), level.to(torch.int64) + half)
+        assert torch.equal(hat, (butterflies(level * sf, order) * rs * sg + P).to(hat.dtype))
+
+
+@pytest.mark.parametrize("d,h,dtype", [(512, 512, synth.F16), (1024, 128, synth.BF16)])
+def test_four_dimensional_reconstruction(d, h, dtype):
+    grid = synth.lloyd_grid(256, seed=7, n_samples=1 << 14, iters=20, dim=4)
+    codec, g = make(d, h, d, dtype, grid), torch.from_numpy(grid).to(DEV)
+    for role in (0, 1):
+        X, prev, W, P = rows(codec, d, dtype, 80 + 10 * role)
+        codes, scales, hat = both_ways(codec, X, prev, W, role)
+        x = butterflies(g[codes.long()].reshape(T, d), range(h.bit_length() - 1)) * rsqrt(h) * signs(d, role)
+        assert torch.equal(hat, fma(x, scales.float(), P).to(hat.dtype))
