@@ -4,6 +4,7 @@ by stage, the normalisation, the search and the reconstruction, restated here wi
 A packed cache outlives the build that wrote it, and a chain of layers passes every moved last bit on to codes of the layers
 that follow, so the order is part of what the library promises and not only the accuracy, which the oracle
 tests check.  The prediction is the library's own (aquakv_predict)."""
+import numpy as np
 import pytest
 import torch
 
@@ -109,12 +110,57 @@ def test_uniform_levels_after_a_rotation(d, h, g, levels, dtype):
         assert torch.equal(hat, (butterflies(level * sf, order) * rs * sg + P).to(hat.dtype))
 
 
-@pytest.mark.parametrize("d,h,dtype", [(512, 512, synth.F16), (1024, 128, synth.BF16)])
-def test_four_dimensional_reconstruction(d, h, dtype):
+def nearest4(y, g):
+    """Index of the point whose half squared distance (less the tuple's own) is the smallest, the first of equal ones."""
+    half = torch.zeros(g.shape[0], device=DEV)
+    for k in range(4):
+        half = fma(g[:, k], g[:, k], half)
+    s = (0.5 * half).expand(y.shape[0], -1)
+    for k in range(4):
+        s = fma(-y[:, k:k + 1], g[:, k], s)
+    return s.argmin(-1)
+
+
+@pytest.mark.parametrize("d,h,dtype", [(512, 512, synth.F16), (1024, 128, synth.BF16), (256, 64, synth.BF16)])
+def test_four_dimensional_grid(d, h, dtype):
     grid = synth.lloyd_grid(256, seed=7, n_samples=1 << 14, iters=20, dim=4)
     codec, g = make(d, h, d, dtype, grid), torch.from_numpy(grid).to(DEV)
+    order = range(h.bit_length() - 1)
     for role in (0, 1):
         X, prev, W, P = rows(codec, d, dtype, 80 + 10 * role)
         codes, scales, hat = both_ways(codec, X, prev, W, role)
-        x = butterflies(g[codes.long()].reshape(T, d), range(h.bit_length() - 1)) * rsqrt(h) * signs(d, role)
-        assert torch.equal(hat, fma(x, scales.float(), P).to(hat.dtype))
+        sg, rs, r = signs(d, role), rsqrt(h), X.float() - P
+        # the scale: eight values a lane, the 32 lanes of a chunk by halving distances, the chunks in order
+        part, total = torch.zeros((T, d // 256, 32), device=DEV), torch.zeros(T, device=DEV)
+        for i in range(8):
+            v = r.view(T, d // 256, 32, 8)[..., i]
+            part = fma(v, v, part)
+        for off in (1, 2, 4, 8, 16):
+            part = part + part[..., torch.arange(32, device=DEV) ^ off]
+        for c in range(d // 256):
+            total = total + part[:, c, 0]
+        assert torch.equal((total * (1.0 / d)).sqrt().half()[:, None], scales)
+        sf = scales.float()
+        y = butterflies(r * (1.0 / sf) * sg, order) * rs
+        q = torch.cat([nearest4(t, g) for t in y.view(-1, 4).split(4096)]).view(T, -1)
+        assert torch.equal(codes.long(), q)
+        assert torch.equal(hat, fma(butterflies(g[q].reshape(T, d), order) * rs * sg, sf, P).to(hat.dtype))
+
+
+def test_four_dimensional_ties_are_decided_by_the_roundings():
+    """Rows of +-1 have scale 1 and rotate to multiples of 1/4; half of the points are the others mirrored in the plane
+    y_k = 1/4, so that many tuples are equally far from two points and the order of the roundings chooses."""
+    d, h = 256, 64
+    rng = np.random.default_rng(3)
+    g = rng.standard_normal((128, 4)).astype(np.float32)
+    m = g.copy()
+    k = np.arange(128)
+    m[k, k % 4] = np.float32(0.5) - g[k, k % 4]
+    grid = np.concatenate([g, m])[rng.permutation(256)]
+    codec = make(d, h, d, synth.BF16, grid)
+    X = torch.from_numpy(rng.choice([-1.0, 1.0], size=(T, d))).to(DEV, torch.bfloat16)
+    codes, scales, _ = codec.encode_phase(0, X)
+    assert bool((scales == 1.0).all())
+    y = butterflies(X.float() * signs(d, 0), range(6)) * 0.125
+    q = torch.cat([nearest4(t, torch.from_numpy(grid).to(DEV)) for t in y.view(-1, 4).split(4096)]).view(T, -1)
+    assert torch.equal(codes.long(), q)
