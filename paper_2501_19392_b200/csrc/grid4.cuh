@@ -105,12 +105,25 @@ __global__ void __launch_bounds__(256) grid4_table_kernel(const float4* __restri
       }
     };
     double U = 1.0e300;
+    int nearest = 0;
     for (int p = 0; p < 256; ++p) {
       double dmin, dmax;
       bounds(p, dmin, dmax);
-      U = fmin(U, dmax);
+      if (dmax < U) {
+        U = dmax;
+        nearest = p;
+      }
     }
-    const double limit = U * (1.0 + 1e-4) + 1e-6;
+    // Two evaluations of grid4_score in single precision are off by at most 16 roundings of its terms, so the distances
+    // they compare by 32 units of 2^-24 of half a point's square plus its largest product with a tuple of the cell:
+    // a point is left out only if it loses by more (twice that, at least 1e-5).
+    auto slack = [&](int p) {
+      const double c[4] = {double(g[p].x), double(g[p].y), double(g[p].z), double(g[p].w)};
+      double terms = 0.0;
+      for (int k = 0; k < 4; ++k) terms += 0.5 * c[k] * c[k] + fabs(c[k]) * fmax(fabs(lo[k]), fabs(hi[k]));
+      return 1e-5 + 4e-6 * terms;
+    };
+    const double limit = U * (1.0 + 1e-4) + 1e-6, slack_u = slack(nearest);
     // candidates by distance, then without those that another one beats everywhere in the cell
     constexpr int kMost = 96;
     unsigned char cand[kMost];
@@ -118,7 +131,7 @@ __global__ void __launch_bounds__(256) grid4_table_kernel(const float4* __restri
     for (int p = 0; p < 256 && m <= kMost; ++p) {
       double dmin, dmax;
       bounds(p, dmin, dmax);
-      if (dmin <= limit) {
+      if (dmin <= limit + fmax(slack(p), slack_u)) {
         if (m < kMost) cand[m] = (unsigned char)p;
         ++m;
       }
@@ -128,6 +141,7 @@ __global__ void __launch_bounds__(256) grid4_table_kernel(const float4* __restri
     for (int i = 0; i < (m <= kMost ? m : 0); ++i) {
       const float4 gi = g[cand[i]];
       const double a[4] = {double(gi.x), double(gi.y), double(gi.z), double(gi.w)};
+      const double slack_i = slack(cand[i]);
       bool beaten = false;
       for (int j = 0; j < m && !beaten; ++j) {
         const float4 gj = g[cand[j]];
@@ -135,7 +149,7 @@ __global__ void __launch_bounds__(256) grid4_table_kernel(const float4* __restri
         // max over the cell of |y - g_j|^2 - |y - g_i|^2 = sum_k 2 y_k (a_k - b_k) + b_k^2 - a_k^2
         double most = 0.0;
         for (int k = 0; k < 4; ++k) most += fmax(2.0 * lo[k] * (a[k] - b[k]), 2.0 * hi[k] * (a[k] - b[k])) + b[k] * b[k] - a[k] * a[k];
-        beaten = most < -1e-5;             // by more than the fp32 evaluation can be off
+        beaten = most < -fmax(slack_i, slack(cand[j]));
       }
       if (!beaten) {
         if (n < 15) w[n >> 2] |= unsigned(cand[i]) << (8 * (n & 3));

@@ -164,3 +164,23 @@ def test_four_dimensional_ties_are_decided_by_the_roundings():
     y = butterflies(X.float() * signs(d, 0), range(6)) * 0.125
     q = torch.cat([nearest4(t, torch.from_numpy(grid).to(DEV)) for t in y.view(-1, 4).split(4096)]).view(T, -1)
     assert torch.equal(codes.long(), q)
+
+
+def test_four_dimensional_lists_keep_what_rounding_can_choose():
+    """Points far from the tuples, in pairs that differ by a few units in the last place: single precision cannot tell
+    which of a pair is nearer, so both have to be among a cell's candidates for the search to equal the exhaustive one."""
+    d, h = 256, 64
+    rng = np.random.default_rng(4)
+    g = rng.standard_normal((128, 4))
+    g = (100.0 * g / np.linalg.norm(g, axis=1, keepdims=True)).astype(np.float32)
+    m = g.copy()
+    k = np.arange(128)
+    m[k, k % 4] += (10.0 ** rng.uniform(-5, -3, 128)).astype(np.float32) * rng.choice([-1.0, 1.0], 128).astype(np.float32)
+    grid = np.concatenate([g, m])[rng.permutation(256)]
+    codec = make(d, h, d, synth.BF16, grid)
+    X = synth.random_16bit((T, d), synth.BF16, 6, device=DEV)
+    codes, scales, _ = codec.encode_phase(0, X)
+    r = X.float()
+    y = butterflies(r * (1.0 / scales.float()) * signs(d, 0), range(6)) * 0.125
+    q = torch.cat([nearest4(t, torch.from_numpy(grid).to(DEV)) for t in y.view(-1, 4).split(4096)]).view(T, -1)
+    assert torch.equal(codes.long(), q)
