@@ -123,6 +123,7 @@ class BufferedKVCache:
         The decoded compressed rows of layer l feed layer l + 1's predictors and are dropped afterwards.
         rope_table (Codec.rope_table): the cached keys are pre-RoPE and are rotated by their positions; q[l] must
         be rotated by the caller."""
+        q = [x.contiguous() for x in q]         # several sequences are one call, and a call's queries follow one another
         out = [torch.empty_like(x) for x in q]
         n16 = self.n_uncompressed
         pos16 = None

@@ -214,3 +214,39 @@ def test_copy_rows_moves_strided_blocks_of_many_tensors():
     torch.cuda.synchronize()
     for x, y in zip(src, dst):
         assert torch.equal(y[:, 5:10], x[:, 2:7]) and not y[:, :5].any() and not y[:, 10:].any()
+
+
+def filled_cache(B, ctx, fill, L=2, cfg=5, seed=40):
+    """A cache policy object in the middle of a conversation, with random contents, and queries for it."""
+    from paper_2501_19392_b200 import policy
+    shape = dataclasses.replace(synth.CONFIGS[cfg], n_tokens=B * (ctx + 256), n_layers=L, batch=B)
+    codec, codec0 = make(shape, 16), make(shape, 256)
+    ad = synth.random_adapters(shape, seed=seed, device=DEV)
+    cache = policy.BufferedKVCache(codec, ad, L, B, max_tokens=ctx + 256, device=DEV, first_layer_codec=codec0)
+    for l in range(L):
+        rc = synth.random_cache(dataclasses.replace(shape, n_layers=1, grid_size=256 if l == 0 else 16), seed=seed + 1 + l,
+                                device=DEV, n_layers=1)
+        for mine, theirs in ((cache.Kcodes, rc.Kcodes), (cache.Vcodes, rc.Vcodes), (cache.Kscales, rc.Kscales), (cache.Vscales, rc.Vscales)):
+            mine[l].copy_(theirs[0].view(mine[l].shape))
+        cache.K16[l].copy_(synth.random_16bit(tuple(cache.K16[l].shape), shape.dtype, seed + 10 + l, device=DEV))
+        cache.V16[l].copy_(synth.random_16bit(tuple(cache.V16[l].shape), shape.dtype, seed + 20 + l, device=DEV))
+    cache.ctx, cache.fill, cache.n_sinks_held = ctx, fill, cache.n_sink
+    q = [synth.random_16bit((B, shape.n_q_heads, shape.head_dim), shape.dtype, seed + 30 + l, device=DEV) for l in range(L)]
+    return cache, shape, q
+
+
+@pytest.mark.parametrize("rope", [False, True])
+def test_queries_that_do_not_follow_one_another(rope):
+    """The last position of [batch, positions, heads, head_dim] queries: dense within a sequence, apart between sequences."""
+    cache, shape, q = filled_cache(3, 200, 40)
+    table = cache.codec.rope_table(shape.head_dim, 5e5, 400, DEV) if rope else None
+    scale = 1.0 / math.sqrt(shape.head_dim)
+    ref = cache.attend(q, shape.n_kv_heads, scale, rope_table=table)
+    apart = []
+    for x in q:
+        big = torch.full((x.shape[0], 5, *x.shape[1:]), 7.0, dtype=x.dtype, device=DEV)
+        big[:, -1] = x
+        apart.append(big[:, -1])
+    assert not apart[0].is_contiguous()
+    for r, o in zip(ref, cache.attend(apart, shape.n_kv_heads, scale, rope_table=table)):
+        assert torch.equal(r, o)
