@@ -479,9 +479,14 @@ class Codec:
         """dst[:] = src for every (src, dst) of [batch, rows, d] 16-bit tensors (any strides over batch and rows), all of
         the same batch and row count, in one launch per 64 pairs."""
         pairs = list(pairs)
-        a = (RowCopy * len(pairs))(*[RowCopy(s.data_ptr(), t.data_ptr(), s.stride(1), s.stride(0), t.stride(1), t.stride(0))
+        batch, rows = (int(x) for x in pairs[0][1].shape[:2]) if pairs else (0, 0)
+        for x in (x for pair in pairs for x in pair):
+            if x.shape != (batch, rows, self.d) or x.stride(2) != 1 or x.element_size() != 2:
+                raise ValueError("copy_rows: %s %s where 16-bit rows [%d, %d, %d] are copied"
+                                 % (tuple(x.shape), x.dtype, batch, rows, self.d))
+        pitch = lambda x: x.stride(0) if batch > 1 else 0
+        a = (RowCopy * len(pairs))(*[RowCopy(s.data_ptr(), t.data_ptr(), s.stride(1), pitch(s), t.stride(1), pitch(t))
                                      for s, t in pairs])
-        batch, rows = (int(x) for x in pairs[0][0].shape[:2]) if pairs else (0, 0)
         rc = lib.aquakv_copy_rows(self.h, len(pairs), a, batch, rows, _stream())
         if rc:
             raise AquaKVError(rc, "aquakv_copy_rows")

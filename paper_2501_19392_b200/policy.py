@@ -80,7 +80,9 @@ class BufferedKVCache:
             t += n
 
     def _store(self, K, V, t, n, row):
-        self.codec.copy_rows((x[l][:, t:t + n], y[l][:, row:row + n])
+        if any(x[l].shape[0] < self.B for x in (K, V) for l in range(self.L)):
+            raise IndexError("append: new tokens of fewer than %d sequences" % self.B)
+        self.codec.copy_rows((x[l][:self.B, t:t + n], y[l][:, row:row + n])
                              for x, y in ((K, self.K16), (V, self.V16)) for l in range(self.L))
 
     def _flush(self):
