@@ -452,11 +452,22 @@ class Codec:
         batch, n_q_heads, head_dim = q.shape
         if out is None:
             out = torch.empty_like(q)
+        if not q.is_contiguous() or not out.is_contiguous():
+            raise ValueError("decode_attn_cache: q and out have to be contiguous")
+        ld16, pitch16 = self.d, n16
+        if K16 is not None or V16 is not None:
+            if K16 is None or V16 is None or K16.shape != V16.shape or K16.stride() != V16.stride():
+                raise ValueError("decode_attn_cache: K16 and V16 have to have the same shape and strides")
+            ld16 = int(K16.stride(1))
+            if batch > 1:
+                pitch16 = int(K16.stride(0)) // max(ld16, 1)
+            if (K16.shape[0] != batch or not n16 <= K16.shape[1] or K16.shape[2] != self.d or K16.stride(2) != 1
+                    or (batch > 1 and pitch16 * ld16 != K16.stride(0))):
+                raise ValueError("decode_attn_cache: K16 / V16 %s with strides %s do not hold %d rows of %d sequences a whole "
+                                 "number of rows apart" % (tuple(K16.shape), tuple(K16.stride()), n16, batch))
         size = lib.aquakv_decode_attn_buffered_workspace_bytes if rope_table is None else lib.aquakv_decode_attn_rope_workspace_bytes
         ws = workspace if workspace is not None else self._workspace(
             int(size(self.h, batch, ctx_len, n16, n_q_heads, head_dim)), q.device)
-        ld16 = self.d if K16 is None else int(K16.stride(1))
-        pitch16 = 0 if K16 is None else int(K16.stride(0)) // ld16
         rc = lib.aquakv_decode_attn_cache(self.h, batch, ctx_len, n_q_heads, n_kv_heads, head_dim, softmax_scale,
                                           _ptr(q), _ptr(Kcodes), _ptr(Kscales), _ptr(Vcodes), _ptr(Vscales),
                                           _ptr(Khat_prev), _ptr(Vhat_prev), _ld(Khat_prev, self.d), _ptr(Wk), _ptr(Wv),

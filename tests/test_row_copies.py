@@ -1,4 +1,4 @@
-"""What the binding hands to the batched row copies, without a GPU: the library call is
+"""What the binding hands to the batched row copies and to the attention over a batch's cache, without a GPU: the library call is
 replaced by one that writes down its arguments.  The C entry points get no shapes, so a batch, a row count or a stride that
 does not fit has to be refused here (the kernels would read or write past the end of a tensor)."""
 import types
@@ -90,3 +90,33 @@ def test_copies_that_fit(calls):
     one = torch.zeros((5, 1, D + 3), dtype=torch.bfloat16).transpose(0, 1)[..., :D]     # one sequence: its pitch is never used
     c.copy_rows([(one, rows(1, 5))])
     assert calls[2][1][2][0].pitch_src == 0
+
+
+def attn(q, K16, V16, n16):
+    return make_codec().decode_attn_cache(q, None, None, None, None, 0, 2, 0.1, K16, V16, n16)
+
+
+Q = torch.zeros((2, 4, 128), dtype=torch.bfloat16)
+
+
+@pytest.mark.parametrize("q,K16,V16,n16", [
+    (torch.zeros((2, 8, 128), dtype=torch.bfloat16)[:, :4], rows(2, 9), rows(2, 9), 5),                       # queries apart
+    (Q, rows(2, 9), rows(2, 10)[:, :9], 5),                                                                  # values pitched otherwise
+    (Q, torch.as_strided(rows(40), (2, 9, D), (9 * D + 8, D, 1)), torch.as_strided(rows(40), (2, 9, D), (9 * D + 8, D, 1)), 5),
+    (Q, rows(2, 9), rows(2, 9), 10),                                                                         # more rows than there are
+    (Q, rows(1, 9), rows(1, 9), 5),                                                                          # a sequence is missing
+    (Q, rows(2, 9), None, 5),
+])
+def test_uncompressed_rows_that_do_not_fit(calls, q, K16, V16, n16):
+    with pytest.raises(ValueError):
+        attn(q, K16, V16, n16)
+    assert not calls
+
+
+def test_uncompressed_rows_that_fit(calls):
+    attn(Q, rows(2, 9), rows(2, 9), 5)
+    attn(Q, rows(2, 9)[..., :], rows(2, 9), 0)
+    attn(Q, None, None, 0)
+    wide = torch.zeros((2, 9, 2 * D), dtype=torch.bfloat16)[..., :D]
+    attn(Q, wide, wide, 9)
+    assert [a[1][21:24] for a in calls] == [(5, D, 9), (0, D, 9), (0, D, 0), (9, 2 * D, 9)]
