@@ -507,7 +507,7 @@ int aquakv_gather_rows(aquakv_ctx* ctx, int64_t n_rows, const int64_t* idx, int6
  * the keys, fit the value predictor on the reconstructed keys, encode the values, hand the
  * reconstructions to the next layer) is made of this call and aquakv_encode_phase.
  * Workspace: aquakv_fit_workspace_bytes(ctx, n_tokens, n_inputs) bytes of device memory, owned by the
- * caller, not read after the call's kernels finish.  Asynchronous on cuda_stream.  Errors: the usual
+ * caller, not read after the call's kernels finish; enough for every smaller n_tokens too.  Asynchronous on cuda_stream.  Errors: the usual
  * argument codes and nothing launched; a matrix that is not positive definite (possible only with
  * rate == 0 and dependent inputs) is reported by aquakv_poll_status as AQUAKV_ERR_NUMERIC.
  * d_kv must be a multiple of 256 (AQUAKV_ERR_UNSUPPORTED otherwise).                                */

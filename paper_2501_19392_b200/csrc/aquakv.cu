@@ -40,6 +40,8 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
+constexpr int kFitMaxSlices = 8;      // of the tokens of a calibration (fit_slices)
+
 struct aquakv_ctx {
   aquakv_params p;
   int log_h, log_g, bits, code_bytes, n_groups;
@@ -62,6 +64,7 @@ struct aquakv_ctx {
   int prof_n;                       // pairs recorded since the last read
   cudaEvent_t* prof_ev;             // 2 * kProfMaxPairs events, created when profiling is enabled
   uint8_t* prof_class;              // kernel class of each pair
+  int fit_from[2][kFitMaxSlices + 1];   // calibration: fewest k-blocks that take s slices, by input tensors (fit_slice_table)
 };
 
 namespace {
@@ -576,24 +579,45 @@ struct FitWs {
   int slices;      // parts the tokens are cut into for the normal equations
 };
 
+// Parts that nk k-blocks of tokens are cut into: as many as fill the CTA pairs evenly; a slice of a tile costs its 256 x
+// 256 partial sums written and read (0.5 MB: the time of about a fifth of a k-block over all pairs).
+int fit_slices(int tiles, int pairs, int nk) {
+  int slices = 1;
+  double best = 0.0;
+  for (int s = 1; s <= kFitMaxSlices && s <= nk; ++s) {
+    const double cost = double((tiles * s + pairs - 1) / pairs) * ((nk + s - 1) / s) + 0.2 * tiles * s;
+    if (s == 1 || cost < best) { best = cost; slices = s; }
+  }
+  return slices;
+}
+
+// The fewest k-blocks that take s slices, for every s.  The slices do not grow with the tokens everywhere (155 blocks may
+// take five, 156 two), but a workspace made for the most tokens has to do for fewer, so it has room for the most
+// slices that any token count up to its own takes.  No slice count is first taken beyond 8192 blocks: the costs per
+// block of two counts differ by at least 1/56 or not at all, against partial sums of at most 0.2 * 68 * 8 blocks (6093
+// blocks), and what the roundings to whole blocks then still decide repeats every 840 blocks.
+void fit_slice_table(aquakv_ctx* c) {
+  for (int n_inputs = 1; n_inputs <= 2; ++n_inputs) {
+    int* from = c->fit_from[n_inputs - 1];
+    for (int s = 0; s <= kFitMaxSlices; ++s) from[s] = INT32_MAX;
+    const int tiles = gram_tiles(c->p.d_kv * n_inputs, c->p.d_kv), pairs = c->sm_count / 2 > 0 ? c->sm_count / 2 : 1;
+    for (int nk = 8192; nk >= 1; --nk) from[fit_slices(tiles, pairs, nk)] = nk;
+  }
+}
+
 FitWs fit_ws(const aquakv_ctx* c, int64_t T, int n_inputs) {
   FitWs w;
   const size_t d = size_t(c->p.d_kv);
   w.n = int(d) * n_inputs;
   w.nk = int((T + kBK - 1) / kBK);
-  // as many slices as fill the CTA pairs evenly; a slice of a tile costs its 256 x 256 partial sums written and read
-  // (0.5 MB: the time of about a fifth of a k-block over all pairs)
-  const int tiles = gram_tiles(w.n, int(d)), pairs = c->sm_count / 2 > 0 ? c->sm_count / 2 : 1;
-  w.slices = 1;
-  double best = 0.0;
-  for (int s = 1; s <= 8 && s <= w.nk; ++s) {
-    const double cost = double((tiles * s + pairs - 1) / pairs) * ((w.nk + s - 1) / s) + 0.2 * tiles * s;
-    if (s == 1 || cost < best) { best = cost; w.slices = s; }
-  }
+  w.slices = fit_slices(gram_tiles(w.n, int(d)), c->sm_count / 2 > 0 ? c->sm_count / 2 : 1, w.nk);
+  int room = w.slices;
+  for (int s = w.slices + 1; s <= kFitMaxSlices; ++s)
+    if (c->fit_from[n_inputs - 1][s] <= w.nk) room = s;
   const size_t n = size_t(w.n);
   size_t off = 0;
   auto take = [&](size_t bytes) { const size_t o = off; off += round_up(bytes, 256); return o; };
-  w.p_off = take(size_t(w.slices) * (n + d) * n * sizeof(float));
+  w.p_off = take(size_t(room) * (n + d) * n * sizeof(float));
   w.m_off = take((n + d) * n * sizeof(double));
   w.inv_off = take(n * sizeof(double));
   w.sums_off = take((n + d) * sizeof(double));
@@ -1312,6 +1336,7 @@ int aquakv_create(const aquakv_params* params, const float* grid_host, const int
   bool ok = cudaGetDevice(&c->device) == cudaSuccess;
   ok = ok && cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, c->device) == cudaSuccess;
   if (ok) {
+    fit_slice_table(c);
     void* fn = nullptr;
     cudaDriverEntryPointQueryResult q;
     ok = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &q) == cudaSuccess &&

@@ -236,3 +236,21 @@ def test_argument_errors_and_a_matrix_that_is_not_positive_definite():
     W16, _, _ = codec.fit_predictor(Y, X, None, rate=1e-3)
     torch.cuda.synchronize()
     assert codec.poll_status() == 0 and torch.isfinite(W16.float()).all()
+
+
+@pytest.mark.parametrize("d", [256, 512, 1024])
+def test_a_workspace_for_the_most_tokens_does_for_fewer(d):
+    from paper_2501_19392_b200 import api
+    grid = synth.lloyd_grid(16, seed=7, n_samples=1 << 12, iters=5)
+    codec = api.Codec(d, d, d, grid, synth.BF16, synth.hadamard_signs(d, 11), synth.hadamard_signs(d, 12))
+    counts = list(range(64, 64 * 700, 64)) + [64 * k + 1 for k in (700, 840, 3000, 8191, 8192, 9000, 20000)]
+    for n_in in (1, 2):
+        need = [codec.fit_workspace_bytes(t, n_in) for t in counts]
+        assert all(a <= b for a, b in zip(need, need[1:]))
+    # a pair of counts of which the smaller one is cut into more slices than the larger one
+    more, most = (9920, 9984) if d == 1024 else (64 * 5, 64 * 6)
+    ws = torch.empty(codec.fit_workspace_bytes(most, 1), dtype=torch.uint8, device="cuda")
+    X, Y = (synth.random_16bit((more, d), synth.BF16, s, device="cuda") for s in (1, 2))
+    W, _, _ = codec.fit_predictor(Y, X, workspace=ws)
+    assert torch.equal(W, codec.fit_predictor(Y, X)[0])
+    assert codec.poll_status() == 0
