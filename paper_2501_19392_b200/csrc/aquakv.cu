@@ -1194,6 +1194,9 @@ int run_chain(aquakv_ctx* c, bool encode, int64_t T, int32_t L, const void* cons
   a.log_h = c->log_h;
   a.log_g = c->log_g;
   a.status = c->d_status;
+  bool any_pred = false;
+  size_t passed = 0;       // reconstructions that products of this call read, one buffer each
+  auto pass = [&]() { return reinterpret_cast<uint16_t*>(wsb + ws.hat_off + passed++ * ws.hat_bytes); };
   for (int l = 0; l < L; ++l) {
     ChainLayer& y = a.layer[l];
     y.K = encode ? static_cast<const uint16_t*>(K[l]) : nullptr;
@@ -1215,12 +1218,14 @@ int run_chain(aquakv_ctx* c, bool encode, int64_t T, int32_t L, const void* cons
     y.ldHat = ld_hat;
     // what later products of this call read: both by the next layer's, the keys by this layer's value product
     const bool next = l + 1 < L && Wk[l + 1] != nullptr;
-    if (next || Wk[l] != nullptr) y.Kpass = reinterpret_cast<uint16_t*>(wsb + ws.hat_off + size_t(2 * l) * ws.hat_bytes);
-    if (next) y.Vpass = reinterpret_cast<uint16_t*>(wsb + ws.hat_off + size_t(2 * l + 1) * ws.hat_bytes);
+    if (next || Wk[l] != nullptr) y.Kpass = pass();
+    if (next) y.Vpass = pass();
+    any_pred = any_pred || Wk[l] != nullptr;
   }
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  // predictions and passed-on reconstructions: all ones = not there yet (the last layer passes its keys at most)
-  if (cudaMemsetAsync(wsb, 0xff, ws.hat_off + size_t(2 * L - 1) * ws.hat_bytes, st) != cudaSuccess) return AQUAKV_ERR_CUDA;
+  // What is polled for (predictions and passed-on reconstructions) is preset to all ones = not there yet.  Without predictors
+  // there is nothing of the kind (2048 tokens x 8 layers of encoding at d_kv 1024: 162 us, 186 with the whole scratch preset).
+  if (any_pred && cudaMemsetAsync(wsb, 0xff, ws.hat_off + passed * ws.hat_bytes, st) != cudaSuccess) return AQUAKV_ERR_CUDA;
   const int grid = c->sm_count;
   a.n_ctas_k = grid / 3 > 0 ? grid / 3 : 1;      // the value predictor has twice the weights: three groups each of 16 and 32 CTAs
   if (grid < 2) return AQUAKV_ERR_UNSUPPORTED;

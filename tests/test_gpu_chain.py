@@ -226,3 +226,23 @@ def test_large_calls_run_several_layers_per_launch_and_equal_the_per_layer_calls
     assert codec.poll_status() == 0
     assert torch.equal(bufs3.K[(L - 1) % 2], hats[-1][0]) and torch.equal(bufs3.V[(L - 1) % 2], hats[-1][1])
     assert torch.equal(bufs3.K[(L - 2) % 2], hats[-2][0]) and torch.equal(bufs3.V[(L - 2) % 2], hats[-2][1])
+
+
+def test_only_what_is_polled_for_is_preset():
+    """A call without predictors writes nothing to its workspace, one with a predictor in one layer only the predictions and the three
+    reconstructions that its products read."""
+    shape = dataclasses.replace(synth.CONFIGS[3], n_tokens=100, n_layers=4)
+    codec, _ = make(shape)
+    kv, ad = synth.kv_chain(shape, seed=7200, device=DEV), synth.random_adapters(shape, seed=7201, device=DEV)
+    none = [None] * 4
+    for W in ((none, none), ([None, ad.Wk[1], None, None], [None, ad.Wv[1], None, None])):
+        ws = torch.full((codec.chain_workspace_bytes(100, 4),), 0x5A, dtype=torch.uint8, device=DEV)
+        Kc, Ks, Vc, Vs, Kh, Vh = buffers(codec, 4, 100)
+        codec.encode_chain(kv.K, kv.V, *W, Kc, Ks, Vc, Vs, Khat=Kh, Vhat=Vh, workspace=ws)
+        Kd, Vd = buffers(codec, 4, 100)[4:]
+        codec.decode_chain(Kc, Ks, Vc, Vs, *W, Khat=Kd, Vhat=Vd, workspace=ws)
+        torch.cuda.synchronize()
+        assert codec.poll_status() == 0
+        assert all(torch.equal(x, y) for x, y in zip(Kh + Vh, Kd + Vd))
+        used = 128 + 2 * 100 * codec.d * 8 + 3 * 100 * codec.d * 2 if W[0][1] is not None else 0
+        assert bool((ws[used:] == 0x5A).all())
