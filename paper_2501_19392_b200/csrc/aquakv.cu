@@ -1227,7 +1227,10 @@ int run_chain(aquakv_ctx* c, bool encode, int64_t T, int32_t L, const void* cons
   // there is nothing of the kind (2048 tokens x 8 layers of encoding at d_kv 1024: 162 us, 186 with the whole scratch preset).
   if (any_pred && cudaMemsetAsync(wsb, 0xff, ws.hat_off + passed * ws.hat_bytes, st) != cudaSuccess) return AQUAKV_ERR_CUDA;
   const int grid = c->sm_count;
-  a.n_ctas_k = grid / 3 > 0 ? grid / 3 : 1;      // the value predictor has twice the weights: three groups each of 16 and 32 CTAs
+  // Keys and values are the same work but for the predictors, of which the values' have twice the weights: three groups
+  // each of 16 and 32 CTAs (d_kv 1024).  Without predictors half of the CTAs each (2048 tokens x 8 layers of encoding: 113 us, with a third for the
+  // keys 162; with predictors in seven of the layers 1160 and 1008).
+  a.n_ctas_k = any_pred ? (grid / 3 > 0 ? grid / 3 : 1) : grid / 2;
   if (grid < 2) return AQUAKV_ERR_UNSUPPORTED;
   ProfScope prof(c, st, AQUAKV_KERNEL_CHAIN);
   AQ_DISPATCH_DNB(launch_chain_dnb, &rc, encode, c->device, st, grid, a);
