@@ -453,12 +453,18 @@ def test_values_around_and_beyond_the_search_table(d, h, n):
     bits = int(np.log2(n))
     bad = (unpack_codes(Kc.cpu().numpy(), bits) != unpack_codes(o["codes"], bits)) & (o["margins"] > 1e-4) & rows_ok[:, None]
     assert rows_ok.sum() >= len(ks) // 2 and not bad.any()
-    # and what no cell holds does not leave the tables: a row that is not finite
+    # and what no cell holds does not leave the tables: a row that is not finite.  Every pair of the value's Hadamard block
+    # becomes NaN or infinite, no point is nearer than another and the exhaustive search stays at index 0; the
+    # scale is the largest finite one; the other rows are what they were.
     bad_row = X.clone()
     bad_row[0, 3], bad_row[1, 5], bad_row[2, 7] = float("nan"), float("inf"), float("-inf")
-    codec.encode(bad_row.to(DEV), bad_row.to(DEV))
+    Kc2, Ks2, Vc2, _, Kh2, _ = codec.encode(bad_row.to(DEV), bad_row.to(DEV))
     torch.cuda.synchronize()
     assert codec.poll_status() == 0
+    assert torch.equal(Kc2[3:], Kc[3:]) and torch.equal(Ks2[3:], Ks[3:]) and torch.equal(Kh2[3:], Kh[3:])
+    for c in (Kc2, Vc2):
+        assert not unpack_codes(c[:3].cpu().numpy(), bits)[:, :h // 2].any()
+    assert (Ks2[:3, 0] == 65504.0).all()
 
 
 @pytest.mark.parametrize("d,h,dtype", [(512, 64, synth.F16), (1024, 1024, synth.BF16)])
