@@ -250,3 +250,21 @@ def test_queries_that_do_not_follow_one_another(rope):
     assert not apart[0].is_contiguous()
     for r, o in zip(ref, cache.attend(apart, shape.n_kv_heads, scale, rope_table=table)):
         assert torch.equal(r, o)
+
+
+@pytest.mark.parametrize("rope", [False, True])
+def test_sequences_served_in_several_groups(rope, monkeypatch):
+    """Five sequences in one group, in groups of two, two and one, and one by one (a context longer than a group): the same
+    results bit for bit."""
+    from paper_2501_19392_b200 import policy
+    ctx, outs = 300, []
+    for tokens in (policy.GROUP_TOKENS, 2 * ctx, 2 * ctx + ctx // 2, ctx - 1):
+        monkeypatch.setattr(policy, "GROUP_TOKENS", tokens)
+        cache, shape, q = filled_cache(5, ctx, 40, L=3)        # its own scratch, sized for these groups
+        table = cache.codec.rope_table(shape.head_dim, 5e5, 500, DEV) if rope else None
+        outs.append(cache.attend(q, shape.n_kv_heads, 1.0 / math.sqrt(shape.head_dim), rope_table=table))
+        torch.cuda.synchronize()
+        assert cache.codec.poll_status() == 0 and cache.codec0.poll_status() == 0
+    for other in outs[1:]:
+        for a, b in zip(outs[0], other):
+            assert torch.equal(a, b)
