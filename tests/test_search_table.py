@@ -2,6 +2,10 @@
 never exclude the true nearest point (Section 2: pairs go to the nearest of n fixed points).  Checked
 without a GPU against brute force in float64 on Gaussian points, on points hugging cell borders and
 on points hugging Voronoi edges."""
+import ctypes
+import os
+import subprocess
+
 import numpy as np
 import pytest
 
@@ -80,3 +84,63 @@ def test_table_keeps_the_nearest_point(n):
         if name == "gauss":     # the exhaustive search must stay rare
             assert brute.mean() < (0.02 if n <= 64 else 1e-3), brute.mean()
             assert lvl2.mean() < 0.25, lvl2.mean()
+
+
+@pytest.fixture(scope="module")
+def repack(tmp_path_factory):
+    """search_table_for_kernels (csrc/search_table.h), compiled on its own: built table and lists -> the kernels' copy."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    out = tmp_path_factory.mktemp("search_table")
+    src, lib = str(out / "shim.cpp"), str(out / "shim.so")
+    with open(src, "w") as f:
+        f.write("""#include <cstring>
+#include "search_table.h"
+extern "C" int words() { return aquakv::kSearchTableWords; }
+extern "C" void repack(const float* grid, int n, const uint32_t* built, uint32_t* out) {
+  const auto v = aquakv::search_table_for_kernels(n, aquakv::search_table_spec(grid, n), built);
+  std::memcpy(out, v.data(), v.size() * sizeof(uint32_t));
+}
+""")
+    subprocess.check_call(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-I",
+                           os.path.join(root, "paper_2501_19392_b200", "csrc"), "-o", lib, src])
+    L = ctypes.CDLL(lib)
+
+    def run(grid, table, lists):
+        built = np.zeros(table.size + 4096, dtype=np.uint32)
+        built[:table.size] = table.ravel()
+        flat = np.ascontiguousarray(lists).reshape(-1).view(np.uint32)
+        built[table.size:table.size + flat.size] = flat
+        got = np.zeros(L.words() + 4096, dtype=np.uint32)
+        g = np.ascontiguousarray(grid, dtype=np.float32)
+        p = lambda a: ctypes.c_void_p(a.ctypes.data)
+        L.repack(p(g), len(g), p(built), p(got))
+        return got[:L.words()], got[L.words():], built[table.size:]
+
+    return run
+
+
+@pytest.mark.parametrize("n", [16, 64, 256])
+def test_the_kernels_copy_holds_the_same_candidates(n, repack):
+    """Entry by entry: the candidates as the kernels read them out of an entry (byte offsets of 8-byte points for n <= 64)
+    are those of the built table, cells that are searched in another way say so, and what the clamped cell numbers 64
+    reach (the next row's first cell, and the row behind the last) is searched exhaustively."""
+    from paper_2501_19392_b200 import api
+    grid = synth.lloyd_grid(n, seed=7, n_samples=1 << 14, iters=25)
+    cells, _, table, lists = api.search_table(grid)
+    e, got_lists, built_lists = repack(grid, table, lists)
+    assert np.array_equal(got_lists, built_lists)
+    built, e = table.ravel(), e.astype(np.int64)
+    special = built >= 0xFF000000
+    assert special.any() and not special.all()
+    if n == 256:
+        assert np.array_equal(e[:built.size], built.astype(np.int64))
+        every = lambda x: x == 0xFFFFFFFF
+    else:
+        every = lambda x: (x & 1) == 1
+        assert np.array_equal(every(e[:built.size]), special)
+        shifts = (24, 16, 8) if n == 16 else (0, 6, 12, 18)
+        for k, s in enumerate(shifts):
+            offset = (e[:built.size] >> s) & (0xFF if n == 16 else 0x1F8)
+            assert np.array_equal(offset[~special], 8 * ((built[~special].astype(np.int64) >> (24 - 8 * k)) & 0xFF))
+    assert every(e[built.size:]).all() and e.size >= 64 * 65 + 1
+    assert every(e[np.arange(64) * 64 + 64]).all()            # column 64 of every row
