@@ -254,7 +254,7 @@ int aquakv_decode(aquakv_ctx* ctx, int64_t n_tokens,
  * Algorithm 4; Section 3.3).  A per-layer call of a few tokens is bound by launch and hand-off
  * latency and by a handful of SMs streaming the adapter weights; here every SM streams a share of
  * the weights, the key chain runs ahead of the value chain, and the layers hand over through
- * counters in device memory.
+ * data that their readers poll for, in the workspace.
  *
  * Per-layer arguments are HOST arrays of n_layers DEVICE pointers (read during the call only):
  * K[l], V[l] (encode), Wk[l], Wv[l] (both NULL: layer l has no predictor, e.g. the model's first

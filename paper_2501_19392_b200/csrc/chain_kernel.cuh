@@ -287,8 +287,8 @@ struct ChainSmem {
 // kWarpRows (D = 1024 with Hadamard block = scale group = 1024 only, checked on the host): the
 // one-warp-per-row routines, which keep more rows in flight; otherwise the team routines (D / 256 warps per
 // row, any supported block / group), whose rows finish sooner.  A layer of a small call is a chain of
-// dependent steps, so the host picks the team routines while every row still gets a team at once
-// (64 tokens x 32 layers: 11.5 against 13.9 us per layer when a stage still ended at a counter) and the warp routines beyond.
+// dependent steps, so the host picks the team routines while every row still gets a team at once and the warp routines beyond
+// (run_chain's launch_chain_dnb has the times of both).
 template <bool kEncode, int D, int NPTS, bool kBf16, bool kWarpRows>
 __global__ void __launch_bounds__(kChainThreads, 1) chain_kernel(const __grid_constant__ ChainArgs a) {
   static_assert(!kWarpRows || D == 1024, "one warp per row needs d_kv = 1024");

@@ -72,7 +72,7 @@ constexpr int kCodecThreads = kCodecWarps * 32;
 // into the grid, whose alignment lets one instruction put an offset under the grid's address; the winner is carried as
 // its offset, which becomes the code when the codes are packed.  29 instructions a pair at n = 16, 60 before:
 // with the transposition of rowwarp.cuh 1435 instead of 1880 warp instructions per row of 1024, and 9472 rows encoded
-// (n = 16, with predictor) in 32.5 instead of 39.0 us; the layer kernel on 32768 tokens 424 -> 396 us.
+// (n = 16, with predictor) in 31.3 instead of 39.0 us; the layer kernel on 32768 tokens 424 -> 397 us.
 constexpr int kSearchCells = 64;          // cells per side of the table (see search_table.h)
 constexpr uint32_t kCellBruteDev = 0xFFFFFFFFu;   // n = 256: "search all points" (the largest entry value)
 constexpr uint32_t kCellSpecialDev = 0xFF000000u; // n = 256: entries from here up: second-level list (low 24 bits) or kCellBruteDev

@@ -22,8 +22,8 @@
 // dependent look-ups, and one row in fifteen has such a tuple.
 //
 // What bounds it: the look-ups of candidates at random indices in shared memory (about eleven passes of the
-// shared-memory pipe each) and the latency of the chain around them at four warps per scheduler.  9472 rows of 1024,
-// with predictor: 75 us (171 us with the lists of the first criterion alone and the exhaustive search per lane).
+// shared-memory pipe each; ncu: that pipe 65 % busy, issue slots 39 %) and the latency of the chain around them at four warps per scheduler.  9472 rows of 1024,
+// with predictor: 77 us (171 us with the lists of the first criterion alone and the exhaustive search per lane).
 #pragma once
 
 #include "uniform.cuh"

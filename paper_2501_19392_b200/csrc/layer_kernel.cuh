@@ -56,16 +56,16 @@ template <bool kEncode, bool kWarpRows> constexpr int kLayerStagesT = (kEncode &
 // (codec.cuh): 24 warps at 64 registers.  The register file is split over the SM's four schedulers, so
 // the budget per thread follows from the warps per scheduler: 4 -> 128, 5 -> 96, 6 -> 80 registers.
 //   encoder: its row work is the longer side of the kernel and gains from every resident warp, even at
-//            80 registers (12 / 14 / 16 / 18-20 row warps measured: 1.51 / 1.48 / 1.38 / 1.46-1.48 ms per
-//            131072 tokens);
+//            80 registers (12 / 14 / 16 / 18 / 20 row warps measured: 1.35 / 1.28 / 1.28 / 1.33 / 1.37 ms per
+//            131072 tokens, 361 / 347 / 350 / 356 / 365 us per 32768);
 //   decoder: the GEMM is the longer side; 10 row warps keep the CTA at 16 warps and 128 registers, which
 //            lets a row issue its prediction loads before the look-ups and the rotation (8 / 10 / 12 row
-//            warps: 0.836 / 0.801-0.809 / 0.835 ms per 131072 tokens).
+//            warps: 0.75 / 0.77 / 0.87 ms per 131072 tokens).
 constexpr int kWrEncodeWarps = 16;
 constexpr int kWrDecodeWarps = 10;
 constexpr int kWrAttnDecodeWarps = 6;  // beside four attention warps: again 16 warps and 128 registers, which the
-                                       // attention warps need as much as the row warps (4 / 5 / 6 / 7 / 10 row warps:
-                                       // 2.19 / 2.07 / 2.07 / 2.35 / 2.22 ms per 8 x 32768 tokens)
+                                       // attention warps need as much as the row warps (4 / 5 / 6 / 7 row warps:
+                                       // 2.54 / 2.41 / 2.23 / 2.94 ms per 8 x 32768 tokens)
 static_assert(kWrAttnDecodeWarps <= kWrDecodeWarps, "the decoder's shared memory is sized for kWrDecodeWarps row warps");
 template <bool kEncode, int D, bool kFull, int kAttnHD = 0>
 struct LayerGeom {
