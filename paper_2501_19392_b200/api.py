@@ -458,13 +458,12 @@ class Codec:
         if K16 is not None or V16 is not None:
             if K16 is None or V16 is None or K16.shape != V16.shape or K16.stride() != V16.stride():
                 raise ValueError("decode_attn_cache: K16 and V16 have to have the same shape and strides")
-            ld16 = int(K16.stride(1))
+            (b16, room, d16), (pitch, ld16, s2) = K16.shape, K16.stride()
             if batch > 1:
-                pitch16 = int(K16.stride(0)) // max(ld16, 1)
-            if (K16.shape[0] != batch or not n16 <= K16.shape[1] or K16.shape[2] != self.d or K16.stride(2) != 1
-                    or (batch > 1 and pitch16 * ld16 != K16.stride(0))):
+                pitch16 = pitch // max(ld16, 1)
+            if b16 != batch or n16 > room or d16 != self.d or s2 != 1 or (batch > 1 and pitch16 * ld16 != pitch):
                 raise ValueError("decode_attn_cache: K16 / V16 %s with strides %s do not hold %d rows of %d sequences a whole "
-                                 "number of rows apart" % (tuple(K16.shape), tuple(K16.stride()), n16, batch))
+                                 "number of rows apart" % (tuple(K16.shape), K16.stride(), n16, batch))
         size = lib.aquakv_decode_attn_buffered_workspace_bytes if rope_table is None else lib.aquakv_decode_attn_rope_workspace_bytes
         ws = workspace if workspace is not None else self._workspace(
             int(size(self.h, batch, ctx_len, n16, n_q_heads, head_dim)), q.device)
@@ -490,14 +489,18 @@ class Codec:
         """dst[:] = src for every (src, dst) of [batch, rows, d] 16-bit tensors (any strides over batch and rows), all of
         the same batch and row count, in one launch per 64 pairs."""
         pairs = list(pairs)
-        batch, rows = (int(x) for x in pairs[0][1].shape[:2]) if pairs else (0, 0)
-        for x in (x for pair in pairs for x in pair):
-            if x.shape != (batch, rows, self.d) or x.stride(2) != 1 or x.element_size() != 2:
-                raise ValueError("copy_rows: %s %s where 16-bit rows [%d, %d, %d] are copied"
-                                 % (tuple(x.shape), x.dtype, batch, rows, self.d))
-        pitch = lambda x: x.stride(0) if batch > 1 else 0
-        a = (RowCopy * len(pairs))(*[RowCopy(s.data_ptr(), t.data_ptr(), s.stride(1), pitch(s), t.stride(1), pitch(t))
-                                     for s, t in pairs])
+        shape = pairs[0][1].shape if pairs else (0, 0, self.d)
+        batch, rows = int(shape[0]), int(shape[1])
+        a = (RowCopy * len(pairs))()
+        for c, (s, t) in zip(a, pairs):
+            si, ti = s.stride(), t.stride()
+            if (s.shape != shape or t.shape != shape or shape[2] != self.d or si[2] != 1 or ti[2] != 1
+                    or s.element_size() != 2 or t.element_size() != 2):
+                raise ValueError("copy_rows: %s %s to %s %s where 16-bit rows [%d, %d, %d] are copied"
+                                 % (tuple(s.shape), s.dtype, tuple(t.shape), t.dtype, batch, rows, self.d))
+            c.src, c.dst, c.ld_src, c.ld_dst = s.data_ptr(), t.data_ptr(), si[1], ti[1]
+            if batch > 1:                    # the pitch of a single sequence is never used
+                c.pitch_src, c.pitch_dst = si[0], ti[0]
         rc = lib.aquakv_copy_rows(self.h, len(pairs), a, batch, rows, _stream())
         if rc:
             raise AquaKVError(rc, "aquakv_copy_rows")

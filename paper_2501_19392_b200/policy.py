@@ -80,10 +80,16 @@ class BufferedKVCache:
             t += n
 
     def _store(self, K, V, t, n, row):
-        if any(x[l].shape[0] < self.B for x in (K, V) for l in range(self.L)):
-            raise IndexError("append: new tokens of fewer than %d sequences" % self.B)
-        self.codec.copy_rows((x[l][:self.B, t:t + n], y[l][:, row:row + n])
-                             for x, y in ((K, self.K16), (V, self.V16)) for l in range(self.L))
+        pairs = []
+        for x, y in ((K, self.K16), (V, self.V16)):
+            for l in range(self.L):
+                new = x[l]
+                if len(new) != self.B:
+                    if len(new) < self.B:
+                        raise IndexError("append: new tokens of fewer than %d sequences" % self.B)
+                    new = new[:self.B]
+                pairs.append((new[:, t:t + n], y[l][:, row:row + n]))
+        self.codec.copy_rows(pairs)
 
     def _flush(self):
         """Compresses the oldest `chunk` rows of the recent buffer (all layers) and closes the gap."""
@@ -140,19 +146,20 @@ class BufferedKVCache:
             self._dec, self._dec_cache = chain.PingPong(self.codec, rows, self.dev), self._compact_cache(rows)
         for b in range(0, self.B, group):
             bs = slice(b, min(b + group, self.B))
+            of = lambda x: x if len(x) == group == self.B else x[bs]        # a tensor's part for these sequences
             n = (bs.stop - b) * self.ctx
             for l in range(self.L):
                 cur, prv = l % 2, (l + 1) % 2
                 has, dec = l > 0 and n > 0, self._dec if n > 0 else None
                 cdc = self.codec0 if l == 0 else self.codec
-                cache = [x[l][bs] for x in (self.Kcodes, self.Kscales, self.Vcodes, self.Vscales)]
+                cache = [of(x[l]) for x in (self.Kcodes, self.Kscales, self.Vcodes, self.Vscales)]
                 if bs.stop - b > 1 and n > 0:       # one sequence's rows are compact as they are
                     cdc.copy_cache(cache, self._dec_cache, bs.stop - b, self.ctx, self.max_ctx, self.ctx)
                     cache = self._dec_cache
                 cdc.decode_attn_cache(
-                    q[l][bs], *cache, self.ctx, n_kv_heads, softmax_scale, self.K16[l][bs] if n16 else None,
-                    self.V16[l][bs] if n16 else None, n16, rope_table, self.n_sinks_held, pos16,
+                    of(q[l]), *cache, self.ctx, n_kv_heads, softmax_scale, of(self.K16[l]) if n16 else None,
+                    of(self.V16[l]) if n16 else None, n16, rope_table, self.n_sinks_held, pos16,
                     dec.K[prv][:n] if has else None, dec.V[prv][:n] if has else None, self.ad.Wk[l] if has else None,
                     self.ad.Wv[l] if has else None, self.ad.bk[l] if has else None, self.ad.bv[l] if has else None,
-                    out=out[l][bs], Khat=dec.K[cur][:n] if dec else None, Vhat=dec.V[cur][:n] if dec else None)
+                    out=of(out[l]), Khat=dec.K[cur][:n] if dec else None, Vhat=dec.V[cur][:n] if dec else None)
         return out
