@@ -133,20 +133,21 @@ class BufferedKVCache:
         be rotated by the caller."""
         q = [x.contiguous() for x in q]         # several sequences are one call, and a call's queries follow one another
         out = [torch.empty_like(x) for x in q]
+        B = min(self.B, len(q[0]))              # queries of the first sequences only are served
         n16 = self.n_uncompressed
         pos16 = None
         if rope_table is not None and n16:
             first_recent = self.n_sinks_held + self.ctx
             pos16 = torch.cat([torch.arange(self.n_sinks_held, dtype=torch.int32, device=self.dev),
                                torch.arange(first_recent, first_recent + self.fill, dtype=torch.int32, device=self.dev)])
-        group = max(1, min(self.B, GROUP_TOKENS // max(self.ctx, 1)))      # sequences decoded together
+        group = max(1, min(B, GROUP_TOKENS // max(self.ctx, 1)))      # sequences decoded together
         if self.ctx > 0 and (self._dec is None or self._dec.K[0].shape[0] < group * self.ctx):
             rows = max(self.max_ctx, min(self.B * self.max_ctx, GROUP_TOKENS))      # enough for every later context
             self._dec = self._dec_cache = None                                      # the old buffers make room first
             self._dec, self._dec_cache = chain.PingPong(self.codec, rows, self.dev), self._compact_cache(rows)
-        for b in range(0, self.B, group):
-            bs = slice(b, min(b + group, self.B))
-            of = lambda x: x if len(x) == group == self.B else x[bs]        # a tensor's part for these sequences
+        for b in range(0, B, group):
+            bs = slice(b, min(b + group, B))
+            of = lambda x: x if len(x) == group == B else x[bs]        # a tensor's part for these sequences
             n = (bs.stop - b) * self.ctx
             for l in range(self.L):
                 cur, prv = l % 2, (l + 1) % 2

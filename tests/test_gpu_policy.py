@@ -268,3 +268,19 @@ def test_sequences_served_in_several_groups(rope, monkeypatch):
     for other in outs[1:]:
         for a, b in zip(outs[0], other):
             assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("queries", [2, 4])
+def test_queries_of_fewer_or_more_sequences_than_the_cache_holds(queries, monkeypatch):
+    """Queries of the first sequences are served, whatever the groups, and surplus ones are not looked at."""
+    from paper_2501_19392_b200 import policy
+    cache, shape, q = filled_cache(3, 200, 40)
+    scale = 1.0 / math.sqrt(shape.head_dim)
+    ref = cache.attend(q, shape.n_kv_heads, scale)
+    other = [torch.cat([x, x])[:queries] for x in q]
+    for tokens in (policy.GROUP_TOKENS, 2 * 200, 1):
+        monkeypatch.setattr(policy, "GROUP_TOKENS", tokens)
+        for r, o in zip(ref, cache.attend(other, shape.n_kv_heads, scale)):
+            n = min(3, queries)
+            assert o.shape[0] == queries and torch.equal(r[:n], o[:n])
+    assert cache.codec.poll_status() == 0
