@@ -236,22 +236,30 @@ __device__ __forceinline__ int wave_block_teams(const WaveRows& w, int block, in
   return (n > 0 ? n : 0) * teams;
 }
 
+// Longest pause (ns; nanosleep takes up to twice that) between two polls of a counter.  A call of one wave is a chain of
+// four steps, and each waits for the one before, so what a poll comes late is lost: with 2 us 10 of the 38 us of 1024 tokens
+// encoded at d_kv 512.  With more waves there is other work in the meantime, and polls cost it issue slots and L2.  us at
+// pauses of 2048 / 512 / 256 / 64: 1024 tokens of d_kv 512, two layers there and back 82 / 75 / 76 / 77; 3001 tokens encoded
+// 88 / 83.5 / 83 / 84.5; 32768 tokens encoded 353 / 357 / 359 / 361.
+__device__ __forceinline__ uint32_t poll_pause(int n_waves) { return n_waves > 1 ? 2048u : 256u; }
+
 __device__ __forceinline__ int ld_acquire(const int* p) {
   int v;
   asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
 }
 
-// Spins until *ctr >= target.  Returns false after kWaitLimitNs or if the CTA already aborted.
+// Spins until *ctr >= target.  Returns false after kWaitLimitNs or if the CTA already aborted.  The pause between two polls
+// doubles up to max_pause: see poll_pause.
 __device__ __forceinline__ bool counter_wait_bounded(const int* ctr, int target, volatile int* abort_flag,
-                                                     int* status) {
+                                                     int* status, uint32_t max_pause) {
   if (ld_acquire(ctr) >= target) return true;
   const unsigned long long t0 = global_timer_ns();
   uint32_t spins = 0;
-  uint32_t pause = 64;          // polls cost issue slots the row warps need: back off up to 2 us
+  uint32_t pause = 64;
   while (ld_acquire(ctr) < target) {
     __nanosleep(pause);
-    if (pause < 2048) pause <<= 1;
+    if (pause < max_pause) pause <<= 1;
     if ((++spins & 0x3Fu) == 0) {
       if (*abort_flag) return false;
       if (global_timer_ns() - t0 > kWaitLimitNs) {
@@ -300,6 +308,7 @@ layer_kernel(const __grid_constant__ LayerBatch<kBatch> B) {
   const int ml0 = 2 * (pair / NTN);                 // the pair is active in a wave iff its first block exists
   const int n_blk = pair % NTN;
   const int n_jobs = 2 * a.n_waves;
+  const uint32_t max_pause = poll_pause(a.n_waves);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kLayerStagesT<kEncode, G::WR>; ++s) {
@@ -363,7 +372,7 @@ layer_kernel(const __grid_constant__ LayerBatch<kBatch> B) {
             const LayerArgs& pa = B.layer[l - 1];
             const int pj = ph == 0 ? layer_key_job(wave) : layer_value_job(wave, a.n_waves);
             const int target = wave_block_teams(wave_rows(wave, a.T, a.mw, gridDim.x), ml, gridDim.x, G::TEAMS);
-            if (!counter_wait_bounded(pa.rows_done + pj * a.mw + ml, target, abort_flag, a.status)) {
+            if (!counter_wait_bounded(pa.rows_done + pj * a.mw + ml, target, abort_flag, a.status, max_pause)) {
               ok = false;
               break;
             }
@@ -373,7 +382,7 @@ layer_kernel(const __grid_constant__ LayerBatch<kBatch> B) {
             // the remaining k-blocks read this wave's reconstructed keys, written by row warps
             const int target = wave_block_teams(wave_rows(wave, a.T, a.mw, gridDim.x), ml, gridDim.x, G::TEAMS);
             if (!counter_wait_bounded(a.rows_done + layer_key_job(wave) * a.mw + ml, target, abort_flag,
-                                      a.status)) {
+                                      a.status, max_pause)) {
               ok = false;
               break;
             }
@@ -491,7 +500,7 @@ layer_kernel(const __grid_constant__ LayerBatch<kBatch> B) {
         const int target = wave_block_teams(wave_rows(wave_old, a.T, a.mw, gridDim.x), ml, gridDim.x, G::TEAMS);
         // one thread polls for the four warps; a failed wait has set the abort flag
         if (warp == 2 && lane == 0)
-          counter_wait_bounded(B.layer[lo].rows_done + jo * a.mw + ml, target, abort_flag, a.status);
+          counter_wait_bounded(B.layer[lo].rows_done + jo * a.mw + ml, target, abort_flag, a.status, max_pause);
         named_barrier(1, 128);
         ok = *abort_flag == 0;
       }
@@ -610,7 +619,7 @@ layer_kernel(const __grid_constant__ LayerBatch<kBatch> B) {
         // two buffer pairs), which that layer's attention warps may, in principle, still be reading
         if (l >= 2) {
           if (lane == 0)
-            ok = counter_wait_bounded(B.layer[l - 2].attn_done + wave * a.mw + rb, NTN * kAttnWarps, abort_flag, a.status);
+            ok = counter_wait_bounded(B.layer[l - 2].attn_done + wave * a.mw + rb, NTN * kAttnWarps, abort_flag, a.status, max_pause);
           ok = __shfl_sync(0xffffffffu, ok, 0);
         }
         // the key rows of this wave reuse the ring rows of wave - ring depth: the attention warps must
@@ -618,7 +627,7 @@ layer_kernel(const __grid_constant__ LayerBatch<kBatch> B) {
         if (ok && ph == 0 && a.khat_ring > 0 && wave >= a.khat_ring) {
           if (lane == 0)
             ok = counter_wait_bounded(a.attn_done + (wave - a.khat_ring) * a.mw + rb, NTN * kAttnWarps, abort_flag,
-                                      a.status);
+                                      a.status, max_pause);
           ok = __shfl_sync(0xffffffffu, ok, 0);
         }
       }
@@ -628,12 +637,12 @@ layer_kernel(const __grid_constant__ LayerBatch<kBatch> B) {
         // one thread polls for the team; all its warps must take the same path, so they agree
         // through the abort flag (set by a failed wait) between two barriers
         if (rck.member == 0 && lane == 0)
-          counter_wait_bounded(a.gemm_done + j * a.mw + rb, NTN, abort_flag, a.status);
+          counter_wait_bounded(a.gemm_done + j * a.mw + rb, NTN, abort_flag, a.status, max_pause);
         team_barrier<D>(rck.barrier);
         ok = *abort_flag == 0;
         team_barrier<D>(rck.barrier);
       } else {
-        if (lane == 0) ok = counter_wait_bounded(a.gemm_done + j * a.mw + rb, NTN, abort_flag, a.status);
+        if (lane == 0) ok = counter_wait_bounded(a.gemm_done + j * a.mw + rb, NTN, abort_flag, a.status, max_pause);
         ok = __shfl_sync(0xffffffffu, ok, 0);
       }
       if (ok) {
@@ -739,7 +748,7 @@ layer_kernel(const __grid_constant__ LayerBatch<kBatch> B) {
         bool ok = true;
         if (lane == 0)
           ok = counter_wait_bounded(a.rows_done + layer_value_job(wave, a.n_waves) * a.mw + ml,
-                                    wave_block_teams(wr, ml, gridDim.x, G::TEAMS), abort_flag, a.status);
+                                    wave_block_teams(wr, ml, gridDim.x, G::TEAMS), abort_flag, a.status, max_pause);
         ok = __shfl_sync(0xffffffffu, ok, 0);
         if (!ok) { stop = true; break; }
         const long long blk = (long long)wave * a.mw + ml;       // token block of the call
