@@ -38,6 +38,12 @@ __device__ __forceinline__ void pdl_sync() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// n 16-byte pieces of one 32-bit word.
+__global__ void __launch_bounds__(256) fill_kernel(uint4* __restrict__ p, uint32_t word, size_t n) {
+  pdl_sync();
+  for (size_t i = blockIdx.x * size_t(256) + threadIdx.x; i < n; i += size_t(gridDim.x) * 256) p[i] = make_uint4(word, word, word, word);
+}
+
 __device__ __forceinline__ unsigned long long global_timer_ns() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
