@@ -585,7 +585,7 @@ EncodeWs encode_ws(const aquakv_ctx* c, int64_t T) {
 // calibration of one predictor (calib.cuh)
 // ---------------------------------------------------------------------------------------------
 struct FitWs {
-  size_t p_off, m_off, inv_off, sums_off, ridge_off, flags_off, flags_bytes, total;
+  size_t p_off, m_off, sums_off, ridge_off, flags_off, flags_bytes, total;
   int n;           // input features
   int nk;          // k-blocks of 64 tokens
   int slices;      // parts the tokens are cut into for the normal equations
@@ -631,7 +631,6 @@ FitWs fit_ws(const aquakv_ctx* c, int64_t T, int n_inputs) {
   auto take = [&](size_t bytes) { const size_t o = off; off += round_up(bytes, 256); return o; };
   w.p_off = take(size_t(room) * (n + d) * n * sizeof(float));
   w.m_off = take((n + d) * n * sizeof(double));
-  w.inv_off = take(n * sizeof(double));
   w.sums_off = take((n + d) * sizeof(double));
   w.ridge_off = take(sizeof(double));
   w.flags_bytes = round_up(((n + d) / kFitNB * (n / kFitNB) + 1) * sizeof(int), 256);      // finished tiles, next task
@@ -1583,7 +1582,6 @@ int aquakv_fit_predictor(aquakv_ctx* c, int64_t n_tokens, const void* in0, const
   uint8_t* ws = ws_base(workspace);
   float* P = reinterpret_cast<float*>(ws + w.p_off);
   double* M = reinterpret_cast<double*>(ws + w.m_off);
-  double* inv_diag = reinterpret_cast<double*>(ws + w.inv_off);
   double* sums = reinterpret_cast<double*>(ws + w.sums_off);
   double* ridge = reinterpret_cast<double*>(ws + w.ridge_off);
   int* flags = reinterpret_cast<int*>(ws + w.flags_off);
@@ -1621,9 +1619,9 @@ int aquakv_fit_predictor(aquakv_ctx* c, int64_t n_tokens, const void* in0, const
         cudaFuncSetAttribute(fit_solve_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
       return AQUAKV_ERR_CUDA;
     const int nc = n / kFitNB, nd = d / kFitNB, tasks = nc * (nc + 1) / 2 + nc * nd, back_tasks = nc * nd;
-    pdl_launch(fit_solve_kernel<false>, dim3(tasks < c->sm_count ? tasks : c->sm_count), dim3(kFitThreads), smem, st, M, n, d, inv_diag, flags, c->d_status);
+    pdl_launch(fit_solve_kernel<false>, dim3(tasks < c->sm_count ? tasks : c->sm_count), dim3(kFitThreads), smem, st, M, n, d, flags, c->d_status);
     pdl_launch(fit_solve_kernel<true>, dim3(back_tasks < c->sm_count ? back_tasks : c->sm_count), dim3(kFitThreads), smem, st, 
-        M, n, d, inv_diag, flags + w.flags_bytes / sizeof(int), c->d_status);
+        M, n, d, flags + w.flags_bytes / sizeof(int), c->d_status);
     c->launches += 2;
   }
   // 4. the adapter in its storage type, and the intercept

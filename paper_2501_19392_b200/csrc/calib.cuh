@@ -309,16 +309,20 @@ __global__ void fit_prepare_kernel(const float* __restrict__ P, int slices, int 
 // matrix instructions (61 of the SM's 64 FMA per clock) from double-buffered shared-memory tiles.
 //
 // What bounds it: the chain diagonal tile -> tile below it -> next diagonal tile, n / 64 times; the arithmetic
-// (n^3 / 3 + n^2 d) would take 0.2 ms of the 2048-feature fit.  A launch per step (diagonal block, panel, update of
-// the trailing matrix: three launches per 32 columns) was bound by the same chain with launches in it.
-// d = 1024, forward / back: 467 / 190 us at n = 1024, 936 / 388 us at n = 2048 (29 / 12 us per 64 columns); the
-// launches per step took 2.8 / 5.6 ms for forward and back together.
+// (n^3 / 3 + n^2 d) would take 0.2 ms of the 2048-feature fit.  A step of the chain, by time stamps: flag and tiles 1.8 us, last
+// product 2.4, diagonal tile 10, store and flag 1.1, its tile to the one below 1.3, triangular solve 1.6, store and flag 0.7.
+// d = 1024, n = 1024 and 2048 together: forward 0.92 ms, back 0.42 (with one pivot at a time and solves of a column at a time
+// 1.40 and 0.58; a launch per step of 32 columns 8.4).
 // ---------------------------------------------------------------------------------------------
 constexpr int kFitThreads = 256;
 constexpr int kFitTile = kFitNB * kFitLd;                                  // doubles of a tile in shared memory
+struct FitCholSmem {
+  double2 col[2][kFitNB];                                                  // a step's two columns
+  double pivot[kFitNB], scale[kFitNB];
+};
 struct FitSolveSmem {
   double t[2][2][kFitTile];                                                // [buffer][row tile, column tile]
-  double col[2][kFitNB];
+  FitCholSmem chol;
   int ready;
   int task;
   int abort_flag;
@@ -369,13 +373,26 @@ __device__ __forceinline__ bool fit_wait(const int* f0, const int* f1, volatile 
   return true;
 }
 
-// Cholesky of the 64 x 64 tile in shared memory (lower triangle), result to global memory.  Thread (ty, tx) of 16 x 16
-// owns rows ty + 16 u and columns tx + 16 v in registers; a column travels through shared memory unscaled, so one
-// barrier per column is enough: a[r][c] -= col[r] * (col[c] / pivot), and L[r][p] = col[r] / sqrt(pivot).  The
-// reciprocals of L's diagonal, which the solves multiply by, go to inv_diag.
+// 1 / x for a normal x > 0: the machine's approximation (about 2^-20) and one step of the third-order iteration
+// r (1 + e + e^2), e = 1 - x r, which leaves the rounding errors of its last addition.
+__device__ __forceinline__ double fit_recip(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+
+// Cholesky factor of the 64 x 64 tile in shared memory (lower triangle), in place, its 16 x 16 diagonal blocks replaced
+// by their inverses (all that the solves need of them).  Thread (ty, tx) of 16 x 16 owns rows ty + 16 u and columns tx + 16 v in registers.
+// Two pivots a step: with the columns c0, c1 of the pair as they stand, z = p00 c1 - p10 c0 (p00 times what the first pivot's
+// elimination leaves of c1) and det = p00 p11 - p10^2 (p00 times the second pivot),
+//   a[r][c] -= c0[r] (c0[c] / p00) + (z[r] / p00) (z[c] / det),
+// the two steps of an elimination one pivot at a time with reciprocals that do not wait for one another.  Columns stay
+// unscaled until the end: L = (c0, z / p00) / sqrt(pivot).  Blocks above the diagonal are left out.
+// What bounds it is the chain of a step: columns to shared memory, barrier, a reciprocal, update; one pivot at a time,
+// with the scaling by a double-precision rsqrt in the chain, took 16.2 us a tile, this 10.
 // A pivot that is not positive sets *status (the matrix was not positive definite) and counts as 1.
-__device__ __forceinline__ void fit_chol_tile(const double* t, double (&col)[2][kFitNB], double* out, long long ld, double* inv_diag,
-                                              int* status) {
+__device__ __forceinline__ void fit_chol_tile(double* t, FitCholSmem& cs, int* status) {
   const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
   double a[4][4];
 #pragma unroll
@@ -385,82 +402,134 @@ __device__ __forceinline__ void fit_chol_tile(const double* t, double (&col)[2][
 #pragma unroll
   for (int v0 = 0; v0 < 4; ++v0) {
 #pragma unroll 1
-    for (int q = 0; q < 16; ++q) {
-      const int p = 16 * v0 + q;
-      double* cb = col[q & 1];
-      if (tx == q) {
+    for (int h = 0; h < 8; ++h) {
+      const int p = 16 * v0 + 2 * h;
+      double2* cb = cs.col[h & 1];
+      if ((tx >> 1) == h) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) cb[ty + 16 * u] = a[u][v0];
+        for (int u = v0; u < 4; ++u) reinterpret_cast<double*>(cb + ty + 16 * u)[tx & 1] = a[u][v0];
       }
       __syncthreads();
-      double piv = cb[p];
-      if (!(piv > 0.0)) {
+      double p00 = cb[p].x;
+      const double p10 = cb[p + 1].x, p11 = cb[p + 1].y;
+      if (!(p00 > 0.0)) {
         if (threadIdx.x == 0) atomicExch(status, kStatusNumeric);
-        piv = 1.0;
+        p00 = 1.0;
       }
-      const double s = rsqrt(piv), inv = s * s;      // one special function per column on the chain
-      double cr[4];
+      double det = fma(p00, p11, -(p10 * p10));
+      if (!(det > 0.0)) {
+        if (threadIdx.x == 0) atomicExch(status, kStatusNumeric);
+        det = p00;
+      }
+      const double r0 = fit_recip(p00), rd = fit_recip(det);
+      if (threadIdx.x == 0) {
+        cs.pivot[p] = p00;
+        cs.pivot[p + 1] = det * r0;
+      }
+      double c0[4], y[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) cr[u] = cb[ty + 16 * u];
+      for (int u = v0; u < 4; ++u) {
+        const double2 c = cb[ty + 16 * u];
+        c0[u] = c.x;
+        y[u] = fma(p00, c.y, -(p10 * c.x)) * r0;
+      }
+      if (tx == 2 * h + 1) {
+#pragma unroll
+        for (int u = v0; u < 4; ++u) a[u][v0] = y[u];
+      }
 #pragma unroll
       for (int v = v0; v < 4; ++v) {
-        const double cc = cb[tx + 16 * v] * inv;
+        const double2 c = cb[tx + 16 * v];
+        const double w0 = c.x * r0, w1 = fma(p00, c.y, -(p10 * c.x)) * rd;
+        if (v > v0 || (tx >> 1) > h) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (v > v0 || tx > q) a[u][v] = fma(-cr[u], cc, a[u][v]);
-      }
-      if (tx == q) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (ty + 16 * u >= p) out[(long long)(ty + 16 * u) * ld + p] = (ty + 16 * u == p ? piv : cr[u]) * s;
-        if (ty == 0) inv_diag[p] = s;
+          for (int u = v; u < 4; ++u) a[u][v] = fma(-y[u], w1, fma(-c0[u], w0, a[u][v]));
+        }
       }
     }
   }
+  __syncthreads();
+  if (threadIdx.x < kFitNB) cs.scale[threadIdx.x] = rsqrt(cs.pivot[threadIdx.x]);
+  __syncthreads();
+#pragma unroll
+  for (int v = 0; v < 4; ++v) {
+    const double sc = cs.scale[tx + 16 * v];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (u > v || (u == v && ty > tx)) t[(ty + 16 * u) * kFitLd + tx + 16 * v] = a[u][v] * sc;
+  }
+  __syncthreads();
+  // inverses of the diagonal blocks: thread (block, column) solves L x = e_column (L's diagonal is 1 / scale)
+  double x[16];
+  const int blk = threadIdx.x >> 4, c = threadIdx.x & 15;
+  if (threadIdx.x < kFitNB) {
+    const double* lb = t + (16 * blk) * kFitLd + 16 * blk;
+#pragma unroll
+    for (int r = 0; r < 16; ++r) x[r] = r == c ? 1.0 : 0.0;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      x[k] *= cs.scale[16 * blk + k];
+#pragma unroll
+      for (int r = k + 1; r < 16; ++r) x[r] = fma(-lb[r * kFitLd + k], x[k], x[r]);
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < kFitNB) {
+#pragma unroll
+    for (int r = 0; r < 16; ++r) t[(16 * blk + r) * kFitLd + 16 * blk + c] = x[r];
+  }
+  __syncthreads();
 }
 
-// X op(L) = T for the 64 x 64 tile T and the lower triangular tile L, both in shared memory; X to global memory:
-// op(L) = L^T (columns of X in ascending order) or, kBack, L (descending).  Four neighbouring lanes share a row, lane
-// q of them owns columns q + 4 w.
+// X op(L) = T for eight rows of a 64 x 64 tile: op(L) = L^T or, kBack, L.  `l`: a tile that fit_chol_tile left, in shared
+// memory.  x enters holding T and leaves holding X as accumulators of the fp64 products: x[c][e] of a lane is row lane / 4,
+// column 8 c + 2 (lane % 4) + e.  Sixteen columns at a time: the block's columns times the inverse of L's diagonal block, then
+// their products with L's blocks beside it off the columns still to come.  An accumulator's element e is an A fragment of the
+// columns 2 k + e, so the rows never leave the warp's registers.  (A column at a time, four lanes a row: 6.1 us a tile,
+// this 1.6.)
 template <bool kBack>
-__device__ __forceinline__ void fit_trsm_tile(const double* t, const double* l, const double* inv_diag, double* out, long long ld) {
-  const int row = threadIdx.x >> 2, q = threadIdx.x & 3;
-  double x[16], inv[16];
+__device__ __forceinline__ void fit_trsm_rows(double (&x)[8][2], const double* l, int lane) {
+  const int g = lane >> 2, k2 = (lane & 3) * 2;
+  // element (k, n) of the B fragment for input columns 8 ct + 2 k + e and output columns 8 co + n
+  auto bfrag = [&](int ct, int co, int e) {
+    return kBack ? l[(8 * ct + k2 + e) * kFitLd + 8 * co + g] : l[(8 * co + g) * kFitLd + 8 * ct + k2 + e];
+  };
 #pragma unroll
-  for (int w = 0; w < 16; ++w) {
-    x[w] = t[row * kFitLd + q + 4 * w];
-    inv[w] = __ldcg(inv_diag + q + 4 * w);
+  for (int s = 0; s < 4; ++s) {
+    const int b = kBack ? 6 - 2 * s : 2 * s;          // first of the block's two column tiles
+    double y[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+#pragma unroll
+    for (int o = 0; o < 2; ++o)
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        if (kBack ? i < o : i > o) continue;          // the inverse is lower triangular
+#pragma unroll
+        for (int e = 0; e < 2; ++e) dmma_8x8x4(y[o][0], y[o][1], x[b + i][e], bfrag(b + i, b + o, e));
+      }
+#pragma unroll
+    for (int o = 0; o < 2; ++o)
+#pragma unroll
+      for (int e = 0; e < 2; ++e) x[b + o][e] = y[o][e];
+#pragma unroll
+    for (int ct = 0; ct < 2; ++ct)
+#pragma unroll
+      for (int e = 0; e < 2; ++e)
+#pragma unroll
+        for (int co = 0; co < 8; ++co)
+          if (kBack ? co < b : co > b + 1) dmma_8x8x4(x[co][0], x[co][1], -y[ct][e], bfrag(b + ct, co, e));
   }
-#pragma unroll
-  for (int s = 0; s < kFitNB; ++s) {
-    const int p = kBack ? kFitNB - 1 - s : s;
-    const double xp = __shfl_sync(0xffffffffu, x[p >> 2] * inv[p >> 2], p & 3, 4);
-    if (q == (p & 3)) x[p >> 2] = xp;
-    if constexpr (kBack) {
-#pragma unroll
-      for (int w = 0; w <= (p >> 2); ++w)
-        if (w < (p >> 2) || q < (p & 3)) x[w] = fma(-xp, l[p * kFitLd + q + 4 * w], x[w]);
-    } else {
-#pragma unroll
-      for (int w = p >> 2; w < 16; ++w)
-        if (w > (p >> 2) || q > (p & 3)) x[w] = fma(-xp, l[(q + 4 * w) * kFitLd + p], x[w]);
-    }
-  }
-#pragma unroll
-  for (int w = 0; w < 16; ++w) out[(long long)row * ld + q + 4 * w] = x[w];
 }
 
 // flags: [(n + d) / 64][n / 64] finished tiles, then the task counter; all zero at launch.
 template <bool kBack>
 __global__ void __launch_bounds__(kFitThreads, 1)
-fit_solve_kernel(double* __restrict__ M, int n, int d, double* __restrict__ inv_diag, int* __restrict__ flags,
-                 int* __restrict__ status) {
+fit_solve_kernel(double* __restrict__ M, int n, int d, int* __restrict__ flags, int* __restrict__ status) {
   extern __shared__ __align__(16) uint8_t fit_smem_raw[];
   FitSolveSmem* sm = reinterpret_cast<FitSolveSmem*>(fit_smem_raw);
   const int nc = n / kFitNB, nr = (n + d) / kFitNB;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int wm = (warp >> 2) * 32, wn = (warp & 3) * 16;        // this warp's 32 x 16 part of a tile
   const int g = lane >> 2, j4 = lane & 3;
+  const int row = warp * 8 + g;                                 // this lane's row of the accumulators: a warp owns 8 x 64
   if (threadIdx.x == 0) sm->abort_flag = 0;
   volatile int* abort_flag = &sm->abort_flag;
   pdl_sync();
@@ -482,15 +551,13 @@ fit_solve_kernel(double* __restrict__ M, int n, int d, double* __restrict__ inv_
       i = col + task - first;
     }
     double* Mij = M + ((long long)i * kFitNB) * n + j * kFitNB;
-    double acc[4][2][2];
+    double acc[8][2];
 #pragma unroll
-    for (int mt = 0; mt < 4; ++mt)
-#pragma unroll
-      for (int nt = 0; nt < 2; ++nt) {
-        const double2 v = *reinterpret_cast<const double2*>(Mij + (long long)(wm + mt * 8 + g) * n + wn + nt * 8 + 2 * j4);
-        acc[mt][nt][0] = v.x;
-        acc[mt][nt][1] = v.y;
-      }
+    for (int nt = 0; nt < 8; ++nt) {
+      const double2 v = *reinterpret_cast<const double2*>(Mij + (long long)row * n + nt * 8 + 2 * j4);
+      acc[nt][0] = v.x;
+      acc[nt][1] = v.y;
+    }
     // left-looking update with the tile pairs of step s = 0, 1, ..; the next pair is fetched while one is multiplied
     // (if it exists by then)
     const int steps = kBack ? nc - 1 - j : j;
@@ -522,29 +589,28 @@ fit_solve_kernel(double* __restrict__ M, int n, int d, double* __restrict__ inv_
       const double* tb = !kBack && i == j ? ta : sm->t[s & 1][1];
 #pragma unroll 4
       for (int kk = 0; kk < kFitNB / 4; ++kk) {
-        double av[4], bv[2];
+        const double av = -ta[row * kFitLd + kk * 4 + j4];
+        double bv[8];
 #pragma unroll
-        for (int mt = 0; mt < 4; ++mt) av[mt] = -ta[(wm + mt * 8 + g) * kFitLd + kk * 4 + j4];
+        for (int nt = 0; nt < 8; ++nt)
+          bv[nt] = kBack ? tb[(kk * 4 + j4) * kFitLd + nt * 8 + g] : tb[(nt * 8 + g) * kFitLd + kk * 4 + j4];
 #pragma unroll
-        for (int nt = 0; nt < 2; ++nt)
-          bv[nt] = kBack ? tb[(kk * 4 + j4) * kFitLd + wn + nt * 8 + g] : tb[(wn + nt * 8 + g) * kFitLd + kk * 4 + j4];
-#pragma unroll
-        for (int mt = 0; mt < 4; ++mt)
-#pragma unroll
-          for (int nt = 0; nt < 2; ++nt) dmma_8x8x4(acc[mt][nt][0], acc[mt][nt][1], av[mt], bv[nt]);
+        for (int nt = 0; nt < 8; ++nt) dmma_8x8x4(acc[nt][0], acc[nt][1], av, bv[nt]);
       }
       __syncthreads();                     // buffer s & 1 may be overwritten, sm->ready read by all
     }
     if (stop) break;
-    double* tt = sm->t[0][0];
-#pragma unroll
-    for (int mt = 0; mt < 4; ++mt)
-#pragma unroll
-      for (int nt = 0; nt < 2; ++nt)
-        *reinterpret_cast<double2*>(tt + (wm + mt * 8 + g) * kFitLd + wn + nt * 8 + 2 * j4) = make_double2(acc[mt][nt][0], acc[mt][nt][1]);
     if (!kBack && i == j) {
+      double* tt = sm->t[0][0];
+#pragma unroll
+      for (int nt = 0; nt < 8; ++nt)
+        *reinterpret_cast<double2*>(tt + row * kFitLd + nt * 8 + 2 * j4) = make_double2(acc[nt][0], acc[nt][1]);
       __syncthreads();
-      fit_chol_tile(tt, sm->col, Mij, n, inv_diag + j * kFitNB, status);
+      fit_chol_tile(tt, sm->chol, status);
+      for (int e = threadIdx.x; e < kFitNB * kFitNB / 2; e += kFitThreads) {
+        const int r = e >> 5, c = (e & 31) * 2;
+        *reinterpret_cast<double2*>(Mij + (long long)r * n + c) = *reinterpret_cast<const double2*>(tt + r * kFitLd + c);
+      }
     } else {
       if (!kBack && threadIdx.x == 0) fit_wait(flags + j * nc + j, flags + j * nc + j, abort_flag, status);
       __syncthreads();
@@ -553,7 +619,10 @@ fit_solve_kernel(double* __restrict__ M, int n, int d, double* __restrict__ inv_
       fit_cp_commit();
       fit_cp_wait_all();
       __syncthreads();
-      fit_trsm_tile<kBack>(tt, sm->t[1][1], inv_diag + j * kFitNB, Mij, n);
+      fit_trsm_rows<kBack>(acc, sm->t[1][1], lane);
+#pragma unroll
+      for (int nt = 0; nt < 8; ++nt)
+        *reinterpret_cast<double2*>(Mij + (long long)row * n + nt * 8 + 2 * j4) = make_double2(acc[nt][0], acc[nt][1]);
     }
     __syncthreads();
     if (threadIdx.x == 0) {                // one releasing thread: the barrier ordered the CTA's stores before its fence
