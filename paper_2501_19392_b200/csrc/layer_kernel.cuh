@@ -19,8 +19,7 @@
 //
 // Dependencies (all counted per job j and token-block slot ml, targets NTN):
 //   gemm_done[j][ml]  -- feature tiles of job j written to the ring        (row warps wait)
-//   rows_done[j][ml]  -- row teams that finished job j on token block ml (target: CTAs per block
-//                        x teams per CTA)                                    (the value-phase TMA
+//   rows_done[j][ml]  -- CTAs whose row teams have finished job j on token block ml (the value-phase TMA
 //                        producer waits for the key rows of its wave; the GEMM epilogue waits for
 //                        job j - ring size before it overwrites that ring slot)
 // Every job waits only on jobs with a smaller index (or the same index of the other role), so the
@@ -86,6 +85,9 @@ constexpr int layer_threads() {
   return LayerGeom<kEncode, D, kFull, kAttnHD>::THREADS + (kAttnHD > 0 ? 32 * kAttnWarps : 0);
 }
 
+// The row warps of a CTA may be a few jobs apart, never kJobRing: a job's predictions wait for the rows of three jobs before.
+constexpr int kJobRing = 8;
+
 struct LayerSmemTail {
   uint64_t full[kLayerStagesMax];
   uint64_t empty[kLayerStagesMax];
@@ -93,6 +95,10 @@ struct LayerSmemTail {
   uint64_t acc_empty[kAccStages];
   uint32_t tmem_base;
   int abort_flag;
+  // hand-offs of the row warps, by job modulo kJobRing; jobs count from 1 through the layers of the launch
+  int poller[kJobRing];      // the latest job that a warp of this CTA polls the GEMM's counter for
+  int ready[kJobRing];       // the latest job whose predictions are there
+  int arrived[kJobRing];     // reports of row teams
 };
 
 // Grid only (decode needs no search table).
@@ -228,20 +234,19 @@ __device__ __forceinline__ WaveRows wave_rows(int wave, int T, int mw, int n_cta
   return w;
 }
 
-// Number of row teams that report on token block `block` of that wave (CTA slots on the block x teams).
-__device__ __forceinline__ int wave_block_teams(const WaveRows& w, int block, int n_ctas, int teams) {
+// Number of CTAs that report on token block `block` of that wave.
+__device__ __forceinline__ int wave_block_ctas(const WaveRows& w, int block, int n_ctas) {
   const int per_block = kBM / w.rpc;
   const int hi = (block + 1) * per_block < n_ctas ? (block + 1) * per_block : n_ctas;
   const int n = hi - block * per_block;
-  return (n > 0 ? n : 0) * teams;
+  return n > 0 ? n : 0;
 }
 
 // Longest pause (ns; nanosleep takes up to twice that) between two polls of a counter.  A call of one wave is a chain of
-// four steps, and each waits for the one before, so what a poll comes late is lost: with 2 us 10 of the 38 us of 1024 tokens
-// encoded at d_kv 512.  With more waves there is other work in the meantime, and polls cost it issue slots and L2.  us at
-// pauses of 2048 / 512 / 256 / 64: 1024 tokens of d_kv 512, two layers there and back 82 / 75 / 76 / 77; 3001 tokens encoded
-// 88 / 83.5 / 83 / 84.5; 32768 tokens encoded 353 / 357 / 359 / 361.
-__device__ __forceinline__ uint32_t poll_pause(int n_waves) { return n_waves > 1 ? 2048u : 256u; }
+// four steps, and each waits for the one before, so what a poll comes late is lost (with pauses of 2 us 10 of the 38 us of 1024
+// tokens encoded at d_kv 512); with more waves there is other work in the meantime.  With one poller per CTA, us at pauses of
+// 2048 / 512 / 256: four sequences of 6017 tokens through four layers of a cache policy 836 / 822 / 819, 5000 tokens decoded 62 / 57 / 56.5.
+__device__ __forceinline__ uint32_t poll_pause(int n_waves) { return n_waves > 1 ? 512u : 128u; }
 
 __device__ __forceinline__ int ld_acquire(const int* p) {
   int v;
@@ -270,6 +275,48 @@ __device__ __forceinline__ bool counter_wait_bounded(const int* ctr, int target,
     }
   }
   return true;
+}
+
+__device__ __forceinline__ int ld_acquire_cta(const int* p) {
+  int v;
+  asm volatile("ld.acquire.cta.shared::cta.s32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
+  return v;
+}
+
+// The row warps' wait for the predictions of job `job` (one lane of each team calls it): the first team of the CTA that
+// comes polls the counter in global memory, the others look at shared memory.  (Every team polling for itself: up to 24
+// pollers in each of 148 CTAs held up the very counters that they waited for.)
+__device__ __forceinline__ bool row_wait(LayerSmemTail* tail, int job, const int* ctr, int target, int* status, uint32_t max_pause) {
+  const int slot = job & (kJobRing - 1);
+  if (ld_acquire_cta(&tail->ready[slot]) >= job) return true;
+  volatile int* abort_flag = &tail->abort_flag;
+  if (atomicMax(&tail->poller[slot], job) < job) {
+    if (!counter_wait_bounded(ctr, target, abort_flag, status, max_pause)) return false;
+    asm volatile("st.release.cta.shared::cta.s32 [%0], %1;" ::"r"(smem_u32(&tail->ready[slot])), "r"(job) : "memory");
+    return true;
+  }
+  const unsigned long long t0 = global_timer_ns();
+  uint32_t spins = 0;
+  while (ld_acquire_cta(&tail->ready[slot]) < job) {
+    __nanosleep(64);
+    if ((++spins & 0xFu) == 0) {
+      if (*abort_flag) return false;
+      if (global_timer_ns() - t0 > 2 * kWaitLimitNs) {       // the polling warp has given up before
+        *abort_flag = 1;
+        atomicExch(status, kStatusTimeout);
+        return false;
+      }
+    }
+  }
+  return true;
+}
+
+// A row team's report on job `job`; true for the last of the CTA's `teams`, which reports for all of them (its fence then
+// covers the rows of the teams that it has synchronised with here).
+__device__ __forceinline__ bool row_arrive(LayerSmemTail* tail, int job, int teams) {
+  int old;
+  asm volatile("atom.acq_rel.cta.shared::cta.add.s32 %0, [%1], 1;" : "=r"(old) : "r"(smem_u32(&tail->arrived[job & (kJobRing - 1)])) : "memory");
+  return (old + 1) % teams == 0;
 }
 
 __device__ __forceinline__ void named_barrier(int id, int threads) {
@@ -320,6 +367,7 @@ layer_kernel(const __grid_constant__ LayerBatch<kBatch> B) {
       mbar_init(&tail->acc_empty[s], 8);     // 4 epilogue warps of each CTA (used in the leader only)
     }
     tail->abort_flag = 0;
+    for (int i = 0; i < kJobRing; ++i) tail->poller[i] = tail->ready[i] = tail->arrived[i] = 0;
     mbar_fence_init();
   }
   if constexpr (kEncode) {
@@ -371,7 +419,7 @@ layer_kernel(const __grid_constant__ LayerBatch<kBatch> B) {
             // the key phase, values for the value phase): its row warps must be done with this token block
             const LayerArgs& pa = B.layer[l - 1];
             const int pj = ph == 0 ? layer_key_job(wave) : layer_value_job(wave, a.n_waves);
-            const int target = wave_block_teams(wave_rows(wave, a.T, a.mw, gridDim.x), ml, gridDim.x, G::TEAMS);
+            const int target = wave_block_ctas(wave_rows(wave, a.T, a.mw, gridDim.x), ml, gridDim.x);
             if (!counter_wait_bounded(pa.rows_done + pj * a.mw + ml, target, abort_flag, a.status, max_pause)) {
               ok = false;
               break;
@@ -380,7 +428,7 @@ layer_kernel(const __grid_constant__ LayerBatch<kBatch> B) {
           }
           if (ph == 1 && kb == NKD && m < a.n_mblocks) {
             // the remaining k-blocks read this wave's reconstructed keys, written by row warps
-            const int target = wave_block_teams(wave_rows(wave, a.T, a.mw, gridDim.x), ml, gridDim.x, G::TEAMS);
+            const int target = wave_block_ctas(wave_rows(wave, a.T, a.mw, gridDim.x), ml, gridDim.x);
             if (!counter_wait_bounded(a.rows_done + layer_key_job(wave) * a.mw + ml, target, abort_flag,
                                       a.status, max_pause)) {
               ok = false;
@@ -497,7 +545,7 @@ layer_kernel(const __grid_constant__ LayerBatch<kBatch> B) {
       }
       if (go >= 0) {
         const int lo = go / n_jobs, jo = go % n_jobs;
-        const int target = wave_block_teams(wave_rows(wave_old, a.T, a.mw, gridDim.x), ml, gridDim.x, G::TEAMS);
+        const int target = wave_block_ctas(wave_rows(wave_old, a.T, a.mw, gridDim.x), ml, gridDim.x);
         // one thread polls for the four warps; a failed wait has set the abort flag
         if (warp == 2 && lane == 0)
           counter_wait_bounded(B.layer[lo].rows_done + jo * a.mw + ml, target, abort_flag, a.status, max_pause);
@@ -637,12 +685,12 @@ layer_kernel(const __grid_constant__ LayerBatch<kBatch> B) {
         // one thread polls for the team; all its warps must take the same path, so they agree
         // through the abort flag (set by a failed wait) between two barriers
         if (rck.member == 0 && lane == 0)
-          counter_wait_bounded(a.gemm_done + j * a.mw + rb, NTN, abort_flag, a.status, max_pause);
+          row_wait(tail, gj + 1, a.gemm_done + j * a.mw + rb, NTN, a.status, max_pause);
         team_barrier<D>(rck.barrier);
         ok = *abort_flag == 0;
         team_barrier<D>(rck.barrier);
       } else {
-        if (lane == 0) ok = counter_wait_bounded(a.gemm_done + j * a.mw + rb, NTN, abort_flag, a.status, max_pause);
+        if (lane == 0) ok = row_wait(tail, gj + 1, a.gemm_done + j * a.mw + rb, NTN, a.status, max_pause);
         ok = __shfl_sync(0xffffffffu, ok, 0);
       }
       if (ok) {
@@ -704,10 +752,9 @@ layer_kernel(const __grid_constant__ LayerBatch<kBatch> B) {
           }
         }
       }
-      // each team reports on its own, so a slow team never holds the others back
       if (TEAM > 1) team_barrier<D>(rck.barrier); else __syncwarp();
       if (*abort_flag) { stop = true; break; }
-      if (rck.member == 0 && lane == 0) {   // one releasing thread per team (see the epilogue)
+      if (rck.member == 0 && lane == 0 && row_arrive(tail, gj + 1, TEAMS)) {   // one releasing thread per CTA (see the epilogue)
         // Key rows are read back by other CTAs' TMA loads (value-phase GEMM) and, like the value rows,
         // by other CTAs' attention warps: those need the stores released, the TMA also across the
         // proxies.  Value rows without attention are read by nobody in this launch; the counter then
@@ -748,7 +795,7 @@ layer_kernel(const __grid_constant__ LayerBatch<kBatch> B) {
         bool ok = true;
         if (lane == 0)
           ok = counter_wait_bounded(a.rows_done + layer_value_job(wave, a.n_waves) * a.mw + ml,
-                                    wave_block_teams(wr, ml, gridDim.x, G::TEAMS), abort_flag, a.status, max_pause);
+                                    wave_block_ctas(wr, ml, gridDim.x), abort_flag, a.status, max_pause);
         ok = __shfl_sync(0xffffffffu, ok, 0);
         if (!ok) { stop = true; break; }
         const long long blk = (long long)wave * a.mw + ml;       // token block of the call
