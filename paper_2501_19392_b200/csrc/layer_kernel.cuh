@@ -40,6 +40,7 @@
 #include "codec.cuh"
 #include "common.cuh"
 #include "gemm_pred.cuh"
+#include "rowchunk.cuh"
 #include "rowwarp.cuh"
 
 namespace aquakv {
@@ -52,7 +53,7 @@ template <bool kEncode, bool kWarpRows> constexpr int kLayerStagesT = (kEncode &
 
 // Row warps of a CTA.  With d_kv = 1024 and the Hadamard block and scale group spanning the whole row
 // (kFull) a single warp owns a row (rowwarp.cuh); otherwise teams of d_kv/256 warps share a row
-// (codec.cuh): 24 warps at 64 registers.  The register file is split over the SM's four schedulers, so
+// (codec.cuh): 24 warps at 64 registers, or, for d_kv <= 512, one warp of rowchunk.cuh.  The register file is split over the SM's four schedulers, so
 // the budget per thread follows from the warps per scheduler: 4 -> 128, 5 -> 96, 6 -> 80 registers.
 //   encoder: its row work is the longer side of the kernel and gains from every resident warp, even at
 //            80 registers (12 / 14 / 16 / 18 / 20 row warps measured: 1.35 / 1.28 / 1.28 / 1.33 / 1.37 ms per
@@ -66,12 +67,21 @@ constexpr int kWrAttnDecodeWarps = 6;  // beside four attention warps: again 16 
                                        // attention warps need as much as the row warps (4 / 5 / 6 / 7 row warps:
                                        // 2.54 / 2.41 / 2.23 / 2.94 ms per 8 x 32768 tokens)
 static_assert(kWrAttnDecodeWarps <= kWrDecodeWarps, "the decoder's shared memory is sized for kWrDecodeWarps row warps");
+enum RowKind { kRowTeams, kRowWarp, kRowChunks };
+// One warp per row for d_kv <= 512 (rowchunk.cuh), row warps by what their registers hold without spills.  us for 60000 tokens:
+//   d_kv 512, Hadamard block and group = the row, encoder: teams 292; 10 / 12 / 14 / 16 warps 257 / 279 / 264 / 299;
+//   d_kv 512, encoder with blocks of 64: teams 264, 10 / 14 warps 282 / 286, so the teams stay;
+//   d_kv 512, decoder: teams 184; 10 / 12 / 14 / 16 warps 178 / 175 / 157 / 167 (blocks of 64: 168; 163 / 159 / 147 / 155);
+//   d_kv 256: 24 / 18 / 16 warps 136 / 128 / 129 to encode and 98 / 88 / 91 to decode, 20000 tokens 63 / - / 59 and 44 / - / 41.
+template <bool kEncode, int D> constexpr int kChunkRowWarps = D == 256 ? 16 : (kEncode ? 10 : 14);
 template <bool kEncode, int D, bool kFull, int kAttnHD = 0>
 struct LayerGeom {
   static constexpr bool WR = D == 1024 && kFull;
-  static constexpr int ROW_WARPS =
-      WR ? (kEncode ? kWrEncodeWarps : (kAttnHD > 0 ? kWrAttnDecodeWarps : kWrDecodeWarps)) : 24;
-  static constexpr int TEAM = WR ? 1 : RowTeam<D>::TEAM;
+  static constexpr bool CR = D == 256 || (D == 512 && (!kEncode || kFull));
+  static constexpr int ROW_WARPS = WR ? (kEncode ? kWrEncodeWarps : (kAttnHD > 0 ? kWrAttnDecodeWarps : kWrDecodeWarps))
+                                      : (CR ? kChunkRowWarps<kEncode, D> : 24);
+  static constexpr int TEAM = WR || CR ? 1 : RowTeam<D>::TEAM;
+  static constexpr int KIND = WR ? kRowWarp : (CR ? kRowChunks : kRowTeams);
   static constexpr int TEAMS = ROW_WARPS / TEAM;          // rows a CTA works on at a time
   static constexpr int THREADS = 32 * (6 + ROW_WARPS);
   // With at most 16 warps per CTA (four per scheduler) a thread may use 128 registers: the row
@@ -109,13 +119,14 @@ struct GridSmem {
 template <bool kEncode, int NPTS> struct LayerTables { typedef RowSmem<NPTS> type; };
 template <int NPTS> struct LayerTables<false, NPTS> { typedef GridSmem<NPTS> type; };
 
-template <int D, int ROW_WARPS, bool WR> struct LayerRowScratch { TeamSmem<D> team[ROW_WARPS / RowTeam<D>::TEAM]; };
-template <int D, int ROW_WARPS> struct LayerRowScratch<D, ROW_WARPS, true> { unsigned long long xbuf[ROW_WARPS][kWrItems]; };
+template <int D, int ROW_WARPS, int kKind> struct LayerRowScratch { TeamSmem<D> team[ROW_WARPS / RowTeam<D>::TEAM]; };
+template <int D, int ROW_WARPS> struct LayerRowScratch<D, ROW_WARPS, kRowWarp> { unsigned long long xbuf[ROW_WARPS][kWrItems]; };
+template <int D, int ROW_WARPS> struct LayerRowScratch<D, ROW_WARPS, kRowChunks> {};
 
 template <bool kEncode, int D, int NPTS, bool kFull>
 struct LayerRowSmem {
   typename LayerTables<kEncode, NPTS>::type tables;
-  LayerRowScratch<D, LayerGeom<kEncode, D, kFull>::ROW_WARPS, LayerGeom<kEncode, D, kFull>::WR> scratch;
+  LayerRowScratch<D, LayerGeom<kEncode, D, kFull>::ROW_WARPS, LayerGeom<kEncode, D, kFull>::KIND> scratch;
 };
 
 // The GEMM epilogue stages each 32-row x 32-column fp32 piece of a tile in shared memory (128-byte
@@ -619,8 +630,16 @@ layer_kernel(const __grid_constant__ LayerBatch<kBatch> B) {
     // one context per warp; the sign bits are switched between key and value jobs
     RowCtx rck;
     WarpRowCtx wrc;
+    ChunkRowCtx crc;
     uint32_t signs_k, signs_v;
-    if constexpr (G::WR) {
+    if constexpr (G::CR) {
+      chunk_ctx_init(crc, log_h, log_g, lane);
+      if constexpr (kEncode) crc.search = search_ctx<NPTS>(&rsm->tables, a.search.inv_w);
+      signs_k = a.signmask_k[lane];
+      signs_v = a.signmask_v[lane];
+      rck.member = 0;
+      rck.barrier = 0;
+    } else if constexpr (G::WR) {
       wrc.lane = lane;
       if constexpr (kEncode) wrc.search = search_ctx<NPTS>(&rsm->tables, a.search.inv_w);
       wrc.signs = 0u;
@@ -643,7 +662,8 @@ layer_kernel(const __grid_constant__ LayerBatch<kBatch> B) {
       const int gj = l * n_jobs + j;
       const WaveRows wr = wave_rows(wave, a.T, a.mw, gridDim.x);
       if (wr.tokens <= 0) continue;
-      if constexpr (G::WR) wrc.signs = ph == 0 ? signs_k : signs_v;
+      if constexpr (G::CR) crc.signs = ph == 0 ? signs_k : signs_v;
+      else if constexpr (G::WR) wrc.signs = ph == 0 ? signs_k : signs_v;
       else row_ctx_set_signs(rck, ph == 0 ? signs_k : signs_v);
       const int slot_row = (ml * NTN + n_blk) * wr.rpc;      // first row (within the wave) of this CTA's slice
       const int rb = slot_row / kBM;                         // token block (within the wave) the slice lies in
@@ -708,7 +728,13 @@ layer_kernel(const __grid_constant__ LayerBatch<kBatch> B) {
           else hat_row = a.Vhat != nullptr ? a.Vhat + g * a.ldVhat : nullptr;
           uint8_t* codes_row = (ph == 0 ? a.Kcodes : a.Vcodes) + g * CODE_BYTES;
           uint16_t* scales_row = (ph == 0 ? a.Kscales : a.Vscales) + g * n_groups;
-          if constexpr (G::WR) {
+          if constexpr (G::CR) {
+            if constexpr (kEncode)
+              chunk_encode_row<D / 256, NPTS, kBf16>(crc, &rsm->tables, (ph == 0 ? a.K : a.V) + g * a.ldX, pred_row, codes_row,
+                                                     scales_row, hat_row);
+            else
+              chunk_decode_row<D / 256, NPTS, kBf16>(crc, rsm->tables.grid, codes_row, scales_row, pred_row, hat_row);
+          } else if constexpr (G::WR) {
             unsigned long long* xbuf = rsm->scratch.xbuf[rw];
             if constexpr (kEncode) {
               const uint16_t* x_row = (ph == 0 ? a.K : a.V) + g * a.ldX;
@@ -740,9 +766,9 @@ layer_kernel(const __grid_constant__ LayerBatch<kBatch> B) {
           // writing them back (the ring is scratch; only whole, 128-byte aligned lines are dropped).
           if (hat_row != nullptr || !kEncode) {
             __syncwarp();
-            if constexpr (G::WR) {
-              const float* mine = pred_row + lane * 32;             // the row's 32 lines, one per lane
-              if ((reinterpret_cast<uintptr_t>(mine) & 127) == 0)
+            if constexpr (G::WR || G::CR) {
+              const float* mine = pred_row + lane * 32;             // the row's lines, one per lane
+              if (lane < D / 32 && (reinterpret_cast<uintptr_t>(mine) & 127) == 0)
                 asm volatile("discard.global.L2 [%0], 128;" ::"l"(mine) : "memory");
             } else {
               const float* mine = pred_row + rck.member * 256 + lane * 8;

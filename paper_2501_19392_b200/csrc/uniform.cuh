@@ -27,6 +27,7 @@
 #pragma once
 
 #include "codec.cuh"
+#include "rowchunk.cuh"
 
 namespace aquakv {
 
@@ -118,35 +119,6 @@ struct UniformRotArgs {
   const uint32_t* signmask;   // [32]: lane's word, bit 8 c + i set where the sign of value 256 c + 8 lane + i is -1
   int log_h;                  // 6 .. 10
 };
-
-template <int NCH>
-__device__ __forceinline__ void row_hadamard(f32x2_t (&v)[NCH][4], int log_h, int lane) {
-#pragma unroll
-  for (int c = 0; c < NCH; ++c) fwht_packed<8>(v[c], log_h, lane);
-#pragma unroll
-  for (int k = 8; k < 10; ++k) {
-    const int m = 1 << (k - 8);
-    if (m < NCH && k < log_h) {
-#pragma unroll
-      for (int c = 0; c < NCH; ++c)
-        if ((c & m) == 0) {
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const f32x2_t a = v[c][i], b = v[c | m][i];
-            v[c][i] = add2(a, b);
-            v[c | m][i] = sub2(a, b);
-          }
-        }
-    }
-  }
-}
-
-// (f, f) with the signs of pair (c, k) of the row: bit 8 c + 2 k and the next of `bits`.
-__device__ __forceinline__ f32x2_t row_signed(float f, uint32_t bits, int c, int k) {
-  const int s = 31 - 8 * c - 2 * k;
-  return pack2(__uint_as_float(__float_as_uint(f) ^ ((bits << s) & 0x80000000u)),
-               __uint_as_float(__float_as_uint(f) ^ ((bits << (s - 1)) & 0x80000000u)));
-}
 
 // The lane's values of row t of the prediction (zeros without one).  kStream: its last read (evict-first); otherwise it
 // stays cached for a second one.
