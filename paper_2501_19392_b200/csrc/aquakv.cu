@@ -937,6 +937,13 @@ int launch_layer(aquakv_ctx* c, cudaStream_t st, bool encode, int64_t T, const v
   if (rc) return rc;
   if ((rc = launch_fill(c, st, B.layer[0].gemm_done, 0u, round_up(ws.flags_bytes, 16)))) return rc;
   const int grid = ws.grid_mw * (d / kBN);
+  B.layer[0].last_log_split = wave_log_split(ws.n_mblocks - (ws.n_waves - 1) * ws.mw, grid / 2, d / kBN);
+  if (B.layer[0].last_log_split > 0) {
+    if ((rc = make_tmap(c, &B.wk_narrow, Wk, uint64_t(d), uint64_t(d), uint64_t(d), kNarrowBox))) return rc;
+    if ((rc = make_tmap(c, &B.wv_narrow, Wv, uint64_t(d), uint64_t(2) * d, uint64_t(2) * d, kNarrowBox))) return rc;
+  } else {
+    B.wk_narrow = B.wv_narrow = B.maps[0].wk;      // not read
+  }
   ProfScope prof(c, st, AQUAKV_KERNEL_LAYER);
   if (encode) {
     AQ_DISPATCH_DNB(launch_layer_enc_t, &rc, c->device, st, grid, B);

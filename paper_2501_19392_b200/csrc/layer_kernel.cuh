@@ -18,7 +18,8 @@
 // a wave (which reads the reconstructed keys of that wave) is issued one job after its key rows.
 //
 // Dependencies (all counted per job j and token-block slot ml, targets NTN):
-//   gemm_done[j][ml]  -- feature tiles of job j written to the ring        (row warps wait)
+//   gemm_done[j][ml]  -- feature tiles of job j written to the ring        (row warps wait; a tile counts kTileWeight, a
+//                        narrow one its part of it)
 //   rows_done[j][ml]  -- CTAs whose row teams have finished job j on token block ml (the value-phase TMA
 //                        producer waits for the key rows of its wave; the GEMM epilogue waits for
 //                        job j - ring size before it overwrites that ring slot)
@@ -158,6 +159,7 @@ struct LayerArgs {
   int n_mblocks;          // ceil(T / 128)
   int mw;                 // token blocks per wave (gridDim.x / NTN)
   int n_waves;
+  int last_log_split;     // wave_log_split of the last wave (launches of one layer)
   int nb;                 // prediction buffers in the ring
   const float* bk;        // optional biases [d_kv]
   const float* bv;
@@ -212,6 +214,15 @@ struct LayerBatch {
   LayerArgs layer[kBatch];
   LayerMaps maps[kBatch];
 };
+// A launch of one layer has room for the maps of narrow tiles: weight boxes of kNarrowBox rows.
+constexpr int kNarrowBox = 32;
+template <>
+struct LayerBatch<1> {
+  int n_layers;
+  LayerArgs layer[1];
+  LayerMaps maps[1];
+  CUtensorMap wk_narrow, wv_narrow;
+};
 static_assert(sizeof(LayerBatch<kLayerBatchMax>) <= 32764, "kernel parameters are limited to 32764 bytes");
 
 __device__ __forceinline__ void layer_job(int j, int n_waves, int& phase, int& wave) {
@@ -219,6 +230,18 @@ __device__ __forceinline__ void layer_job(int j, int n_waves, int& phase, int& w
   else if (j == 2 * n_waves - 1) { phase = 1; wave = n_waves - 1; }
   else if (j & 1) { phase = 0; wave = (j + 1) >> 1; }
   else { phase = 1; wave = (j >> 1) - 1; }
+}
+// log2 of the number of tiles that a 256-feature tile is cut into in the last wave of a call, the only one that may be short.
+// A short wave leaves CTA pairs without a tile, while those that have one take the k-blocks and the pieces of the epilogue
+// (0.5 - 0.7 us per 32 features) one after the other: narrower tiles shorten both.  As many as there are pairs for, up to four (64 features:
+// below that the token rows are most of what a k-block loads).  us with whole and with narrow tiles: 1000 tokens of
+// d_kv 1024 encoded 49.7 / 42.7 and decoded 34.5 / 29.7, 2000 54.8 / 50.7 and 39.2 / 37.2, 5000 (the second wave is short) 86.4 / 83.6
+// and 57.0 / 54.6.  Launches of several layers keep whole tiles: no room for the maps of narrow ones.
+constexpr int kTileWeight = 4;
+inline int wave_log_split(int blocks, int pairs, int ntn) {
+  int ls = 0;
+  while (ls < 2 && ((blocks + 1) / 2 * ntn << (ls + 1)) <= pairs) ++ls;
+  return ls;
 }
 __device__ __forceinline__ int layer_key_job(int wave) { return wave == 0 ? 0 : 2 * wave - 1; }
 __device__ __forceinline__ int layer_value_job(int wave, int n_waves) {
@@ -362,9 +385,25 @@ layer_kernel(const __grid_constant__ LayerBatch<kBatch> B) {
   const int lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();          // 0 = leader of the pair (issues the MMAs)
   const int pair = blockIdx.x >> 1;
-  const int ml = 2 * (pair / NTN) + int(rank);
-  const int ml0 = 2 * (pair / NTN);                 // the pair is active in a wave iff its first block exists
+  const int ml = 2 * (pair / NTN) + int(rank);      // token block and feature tile of this CTA in a full wave
   const int n_blk = pair % NTN;
+  // The GEMM tile of this pair in a wave: token-block slots 2 * (pair / tiles), + 1 and feature tile pair % tiles of `width`
+  // features, tiles = NTN << log_split.
+  struct Tile {
+    int log_split, width, ml, n;
+    bool active;        // the pair's first token block exists
+  };
+  constexpr int LOG_NTN = NTN == 4 ? 2 : (NTN == 2 ? 1 : 0);
+  auto wave_tile = [&](int wave) {
+    Tile t;
+    t.log_split = kBatch == 1 && wave == a.n_waves - 1 ? a.last_log_split : 0;
+    t.width = kBN >> t.log_split;
+    const int log_tiles = LOG_NTN + t.log_split, slot = (pair >> log_tiles) * 2;
+    t.n = pair & ((1 << log_tiles) - 1);
+    t.ml = slot + int(rank);
+    t.active = wave * a.mw + slot < a.n_mblocks && slot < a.mw;
+    return t;
+  };
   const int n_jobs = 2 * a.n_waves;
   const uint32_t max_pause = poll_pause(a.n_waves);
 
@@ -420,10 +459,24 @@ layer_kernel(const __grid_constant__ LayerBatch<kBatch> B) {
       for (int j = 0; ok && j < n_jobs; ++j) {
         int ph, wave;
         layer_job(j, a.n_waves, ph, wave);
-        const int m = wave * a.mw + ml;
-        if (wave * a.mw + ml0 >= a.n_mblocks) continue;
+        const Tile tile = wave_tile(wave);
+        if (!tile.active) continue;
+        const int ml = tile.ml, m = wave * a.mw + ml;
         const int nk = ph == 0 ? NKD : 2 * NKD;
+        const int w_row = tile.n * tile.width + int(rank) * (tile.width / 2);     // this CTA's half of the weight rows
+        const uint32_t stage_tx = 2u * uint32_t(kABytes + (kPairBBytes >> tile.log_split));
         const int khat_row = a.khat_ring ? ((wave % a.khat_ring) * a.mw + ml) * kBM : m * kBM;
+        auto load_weights = [&](uint8_t* dst, const CUtensorMap* whole, int which, int x) {
+          if constexpr (kBatch == 1) {
+            if (tile.log_split > 0) {
+              const CUtensorMap* narrow = which == 0 ? &B.wk_narrow : &B.wv_narrow;
+              for (int r = 0; r < tile.width / 2; r += kNarrowBox)
+                tma_load_2d_pair_hint(dst + r * (kBK * 2), narrow, &tail->full[stage], x, w_row + r, pol_keep);
+              return;
+            }
+          }
+          tma_load_2d_pair_hint(dst, whole, &tail->full[stage], x, w_row, pol_keep);
+        };
         for (int kb = 0; kb < nk; ++kb) {
           if (l > 0 && kb == 0 && m < a.n_mblocks) {
             // the previous layer of this launch wrote this job's first input (its reconstructed keys for
@@ -454,19 +507,18 @@ layer_kernel(const __grid_constant__ LayerBatch<kBatch> B) {
           uint8_t* a_dst = smem + size_t(stage) * kPairStageBytes;
           uint8_t* b_dst = a_dst + kABytes;
           // the leader's barrier collects the bytes of both CTAs
-          if (rank == 0) mbar_arrive_expect_tx(&tail->full[stage], 2 * kPairStageBytes);
-          const int w_row = n_blk * kBN + int(rank) * (kBN / 2);     // this CTA's half of the weight rows
+          if (rank == 0) mbar_arrive_expect_tx(&tail->full[stage], stage_tx);
           // token rows stream through L2 once; the adapter tiles are read again by every wave
           if (ph == 0) {
             tma_load_2d_pair_hint(a_dst, &tm.kprev, &tail->full[stage], kb * kBK, m * kBM, pol_stream);
-            tma_load_2d_pair_hint(b_dst, &tm.wk, &tail->full[stage], kb * kBK, w_row, pol_keep);
+            load_weights(b_dst, &tm.wk, 0, kb * kBK);
           } else {
             if (kb < NKD) {
               tma_load_2d_pair_hint(a_dst, &tm.vprev, &tail->full[stage], kb * kBK, m * kBM, pol_stream);
             } else {
               tma_load_2d_pair_hint(a_dst, &tm.khat, &tail->full[stage], (kb - NKD) * kBK, khat_row, pol_stream);
             }
-            tma_load_2d_pair_hint(b_dst, &tm.wv, &tail->full[stage], kb * kBK, w_row, pol_keep);
+            load_weights(b_dst, &tm.wv, 1, kb * kBK);
           }
           ++issued;
           if (++stage == kLayerStagesT<kEncode, G::WR>) { stage = 0; phase_bit ^= 1u; }
@@ -490,7 +542,6 @@ layer_kernel(const __grid_constant__ LayerBatch<kBatch> B) {
   } else if (warp == 1) {
     // ------------------------------- MMA issuer ----------------------------------------------
     if (lane == 0 && rank == 0) {
-      constexpr uint32_t idesc = umma_idesc_f16(2 * kBM, kBN, kBf16);
       int stage = 0;
       uint32_t phase_bit = 0;
       bool ok = true;
@@ -499,7 +550,9 @@ layer_kernel(const __grid_constant__ LayerBatch<kBatch> B) {
       for (int j = 0; ok && j < n_jobs; ++j) {
         int ph, wave;
         layer_job(j, a.n_waves, ph, wave);
-        if (wave * a.mw + ml0 >= a.n_mblocks) continue;
+        const Tile tile = wave_tile(wave);
+        if (!tile.active) continue;
+        const uint32_t idesc = umma_idesc_f16(2 * kBM, tile.width, kBf16);
         const int nk = ph == 0 ? NKD : 2 * NKD;
         const int acc = it & 1;
         const uint32_t acc_phase = (it >> 1) & 1u;
@@ -538,7 +591,9 @@ layer_kernel(const __grid_constant__ LayerBatch<kBatch> B) {
     for (int j = 0; j < n_jobs; ++j) {
       int ph, wave;
       layer_job(j, a.n_waves, ph, wave);
-      if (wave * a.mw + ml0 >= a.n_mblocks) continue;
+      const Tile tile = wave_tile(wave);
+      if (!tile.active) continue;
+      const int ml = tile.ml, x0 = tile.n * tile.width, n_pieces = tile.width / 32;
       const int acc = it & 1;
       const uint32_t acc_phase = (it >> 1) & 1u;
       ++it;
@@ -574,11 +629,11 @@ layer_kernel(const __grid_constant__ LayerBatch<kBatch> B) {
         const uint64_t pol_keep = l2_policy_evict_last();
         uint8_t* my_epi = epi_smem + (warp - 2) * EB * kEpiPieceBytes;
 #pragma unroll 1
-        for (int c = 0; c < kBN / 32; ++c) {
+        for (int c = 0; c < n_pieces; ++c) {
           float v[32];
           tmem_ld_32x32b_x32(taddr + uint32_t(c * 32), v);
           if (bias != nullptr) {
-            const float* b = bias + n_blk * kBN + c * 32;
+            const float* b = bias + x0 + c * 32;
 #pragma unroll
             for (int i = 0; i < 32; ++i) v[i] = __fadd_rn(v[i], __ldg(b + i));
           }
@@ -597,7 +652,7 @@ layer_kernel(const __grid_constant__ LayerBatch<kBatch> B) {
           fence_proxy_async_smem();
           __syncwarp();
           if (lane == 0) {
-            tma_store_2d_hint(&tm.p, buf, n_blk * kBN + c * 32, ring_row, pol_keep);   // read back soon by the row warps
+            tma_store_2d_hint(&tm.p, buf, x0 + c * 32, ring_row, pol_keep);   // read back soon by the row warps
             bulk_commit();
           }
         }
@@ -616,7 +671,7 @@ layer_kernel(const __grid_constant__ LayerBatch<kBatch> B) {
       if (*abort_flag) { stop = true; break; }
       if (warp == 2 && lane == 0) {
         __threadfence();
-        atomicAdd(a.gemm_done + j * a.mw + ml, 1);
+        atomicAdd(a.gemm_done + j * a.mw + ml, kTileWeight >> tile.log_split);
       }
     }
     }   // layers
@@ -705,12 +760,12 @@ layer_kernel(const __grid_constant__ LayerBatch<kBatch> B) {
         // one thread polls for the team; all its warps must take the same path, so they agree
         // through the abort flag (set by a failed wait) between two barriers
         if (rck.member == 0 && lane == 0)
-          row_wait(tail, gj + 1, a.gemm_done + j * a.mw + rb, NTN, a.status, max_pause);
+          row_wait(tail, gj + 1, a.gemm_done + j * a.mw + rb, kTileWeight * NTN, a.status, max_pause);
         team_barrier<D>(rck.barrier);
         ok = *abort_flag == 0;
         team_barrier<D>(rck.barrier);
       } else {
-        if (lane == 0) ok = row_wait(tail, gj + 1, a.gemm_done + j * a.mw + rb, NTN, a.status, max_pause);
+        if (lane == 0) ok = row_wait(tail, gj + 1, a.gemm_done + j * a.mw + rb, kTileWeight * NTN, a.status, max_pause);
         ok = __shfl_sync(0xffffffffu, ok, 0);
       }
       if (ok) {
