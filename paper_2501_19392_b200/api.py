@@ -50,6 +50,9 @@ class AquaKVError(RuntimeError):
         super().__init__("%s failed: %d (%s)" % (where, status, status_string(status)))
 
 
+_POINTERS = {}      # array types by length: making one for every argument was a third of a chain call's host time
+
+
 class RowCopy(ctypes.Structure):
     _fields_ = [("src", ctypes.c_void_p), ("dst", ctypes.c_void_p), ("ld_src", ctypes.c_int64),
                 ("pitch_src", ctypes.c_int64), ("ld_dst", ctypes.c_int64), ("pitch_dst", ctypes.c_int64)]
@@ -536,7 +539,13 @@ class Codec:
         if tensors is None:
             return None
         assert len(tensors) == n
-        return (ctypes.c_void_p * n)(*[_ptr(t) for t in tensors])
+        array = _POINTERS.get(n)
+        if array is None:
+            array = _POINTERS[n] = ctypes.c_void_p * n
+        try:
+            return array(*[None if t is None else t.data_ptr() for t in tensors])
+        except AttributeError:          # plain addresses among them
+            return array(*[_ptr(t) for t in tensors])
 
     def chain_workspace_bytes(self, n_tokens: int, n_layers: int) -> int:
         return int(lib.aquakv_chain_workspace_bytes(self.h, n_tokens, n_layers))
