@@ -373,24 +373,17 @@ __device__ __forceinline__ bool fit_wait(const int* f0, const int* f1, volatile 
   return true;
 }
 
-// 1 / x for a normal x > 0: the machine's approximation (about 2^-20) and one step of the third-order iteration
-// r (1 + e + e^2), e = 1 - x r, which leaves the rounding errors of its last addition.
-__device__ __forceinline__ double fit_recip(double x) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  const double e = fma(-x, r, 1.0);
-  return fma(r, fma(e, e, e), r);
-}
-
 // Cholesky factor of the 64 x 64 tile in shared memory (lower triangle), in place, its 16 x 16 diagonal blocks replaced
 // by their inverses (all that the solves need of them).  Thread (ty, tx) of 16 x 16 owns rows ty + 16 u and columns tx + 16 v in registers.
-// Two pivots a step: with the columns c0, c1 of the pair as they stand, z = p00 c1 - p10 c0 (p00 times what the first pivot's
+// Two pivots a step: with the columns c0, c1 of the pair as they stand, m = p10 / p00, y = c1 - m c0 (what the first pivot's
 // elimination leaves of c1) and det = p00 p11 - p10^2 (p00 times the second pivot),
-//   a[r][c] -= c0[r] (c0[c] / p00) + (z[r] / p00) (z[c] / det),
+//   a[r][c] -= c0[r] (c0[c] / p00) + y[r] (y[c] (p00 / det)),
 // the two steps of an elimination one pivot at a time with reciprocals that do not wait for one another.  Columns stay
-// unscaled until the end: L = (c0, z / p00) / sqrt(pivot).  Blocks above the diagonal are left out.
-// What bounds it is the chain of a step: columns to shared memory, barrier, a reciprocal, update; one pivot at a time,
-// with the scaling by a double-precision rsqrt in the chain, took 16.2 us a tile, this 10.
+// unscaled until the end: L = (c0, y) / sqrt(pivot).  Blocks above the diagonal are left out.
+// What bounds it is the chain of a step, columns to shared memory, barrier, reciprocals, update, and its double-precision
+// instructions, of which an SM issues two warps' worth a clock at best.  Both reciprocals are one call, the odd lanes with the other argument
+// (two calls: 2 % of a calibration of 32768 tokens, d_kv 1024).  One pivot at a time, with the scaling by a double-precision rsqrt in the
+// chain, took 16.2 us a tile, this 10.
 // A pivot that is not positive sets *status (the matrix was not positive definite) and counts as 1.
 __device__ __forceinline__ void fit_chol_tile(double* t, FitCholSmem& cs, int* status) {
   const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
@@ -421,17 +414,19 @@ __device__ __forceinline__ void fit_chol_tile(double* t, FitCholSmem& cs, int* s
         if (threadIdx.x == 0) atomicExch(status, kStatusNumeric);
         det = p00;
       }
-      const double r0 = fit_recip(p00), rd = fit_recip(det);
+      const double rr = __drcp_rn(threadIdx.x & 1 ? det : p00);
+      const double r0 = __shfl_sync(0xffffffffu, rr, 0), rd = __shfl_sync(0xffffffffu, rr, 1);
       if (threadIdx.x == 0) {
         cs.pivot[p] = p00;
         cs.pivot[p + 1] = det * r0;
       }
+      const double m = p10 * r0, r1 = p00 * rd;
       double c0[4], y[4];
 #pragma unroll
       for (int u = v0; u < 4; ++u) {
         const double2 c = cb[ty + 16 * u];
         c0[u] = c.x;
-        y[u] = fma(p00, c.y, -(p10 * c.x)) * r0;
+        y[u] = fma(-m, c.x, c.y);
       }
       if (tx == 2 * h + 1) {
 #pragma unroll
@@ -440,7 +435,7 @@ __device__ __forceinline__ void fit_chol_tile(double* t, FitCholSmem& cs, int* s
 #pragma unroll
       for (int v = v0; v < 4; ++v) {
         const double2 c = cb[tx + 16 * v];
-        const double w0 = c.x * r0, w1 = fma(p00, c.y, -(p10 * c.x)) * rd;
+        const double w0 = c.x * r0, w1 = fma(-m, c.x, c.y) * r1;
         if (v > v0 || (tx >> 1) > h) {
 #pragma unroll
           for (int u = v; u < 4; ++u) a[u][v] = fma(-y[u], w1, fma(-c0[u], w0, a[u][v]));

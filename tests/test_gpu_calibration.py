@@ -254,3 +254,18 @@ def test_a_workspace_for_the_most_tokens_does_for_fewer(d):
     W, _, _ = codec.fit_predictor(Y, X, workspace=ws)
     assert torch.equal(W, codec.fit_predictor(Y, X)[0])
     assert codec.poll_status() == 0
+
+
+@pytest.mark.parametrize("rate", [1e100, 1e160, 1e300])
+def test_a_ridge_that_outweighs_everything_gives_the_intercept_alone(rate):
+    """W = C / ridge underflows to zero and the intercept is the mean of the targets, however large the rate: products of
+    two diagonal elements (1e324 and more here) must not decide that."""
+    shape = small_shape(2, 300, 2, oracle.BF16)
+    codec, _ = make(shape)
+    X, Y = (synth.random_16bit((300, shape.d_kv), oracle.BF16, s, device=DEV) for s in (1, 2))
+    W16, b, W32 = codec.fit_predictor(Y, X, None, rate=rate, fit_bias=True, want_fp32=True)
+    torch.cuda.synchronize()
+    assert codec.poll_status() == 0
+    assert (W16 == 0).all() and (W32 == 0).all()
+    mean = Y.double().mean(0)
+    assert (b.double() - mean).abs().max() <= 2.0 ** -23 * mean.abs().max()       # rounded once to fp32
