@@ -508,8 +508,9 @@ int aquakv_gather_rows(aquakv_ctx* ctx, int64_t n_rows, const int64_t* idx, int6
  * reconstructions to the next layer) is made of this call and aquakv_encode_phase.
  * Workspace: aquakv_fit_workspace_bytes(ctx, n_tokens, n_inputs) bytes of device memory, owned by the
  * caller, not read after the call's kernels finish; enough for every smaller n_tokens too.  Asynchronous on cuda_stream.  Errors: the usual
- * argument codes and nothing launched; a matrix that is not positive definite (possible only with
- * rate == 0 and dependent inputs) is reported by aquakv_poll_status as AQUAKV_ERR_NUMERIC.
+ * argument codes and nothing launched; a pivot that comes out not positive (possible only with
+ * dependent inputs and a rate that is 0 or lost in the rounding of the sums) is reported by aquakv_poll_status as
+ * AQUAKV_ERR_NUMERIC.  Equal features in columns 2i and 2i + 1 always are; other dependences may hide in the rounding.
  * d_kv must be a multiple of 256 (AQUAKV_ERR_UNSUPPORTED otherwise).                                */
 size_t aquakv_fit_workspace_bytes(const aquakv_ctx* ctx, int64_t n_tokens, int32_t n_inputs);
 int aquakv_fit_predictor(aquakv_ctx* ctx, int64_t n_tokens, const void* in0, const void* in1, int64_t ld_in,

@@ -378,7 +378,8 @@ __device__ __forceinline__ bool fit_wait(const int* f0, const int* f1, volatile 
 // Two pivots a step: with the columns c0, c1 of the pair as they stand, m = p10 / p00, y = c1 - m c0 (what the first pivot's
 // elimination leaves of c1) and det = p00 p11 - p10^2 (p00 times the second pivot),
 //   a[r][c] -= c0[r] (c0[c] / p00) + y[r] (y[c] (p00 / det)),
-// the two steps of an elimination one pivot at a time with reciprocals that do not wait for one another.  Columns stay
+// the two steps of an elimination one pivot at a time with reciprocals that do not wait for one another.  det carries the
+// rounding error of p10^2 along (Kahan's difference of two products), so that it is exactly zero for a feature given twice, p00 = p10 = p11.  Columns stay
 // unscaled until the end: L = (c0, y) / sqrt(pivot).  Blocks above the diagonal are left out.
 // What bounds it is the chain of a step, columns to shared memory, barrier, reciprocals, update, and its double-precision
 // instructions, of which an SM issues two warps' worth a clock at best.  Both reciprocals are one call, the odd lanes with the other argument
@@ -409,7 +410,8 @@ __device__ __forceinline__ void fit_chol_tile(double* t, FitCholSmem& cs, int* s
         if (threadIdx.x == 0) atomicExch(status, kStatusNumeric);
         p00 = 1.0;
       }
-      double det = fma(p00, p11, -(p10 * p10));
+      const double pp = p10 * p10;
+      double det = fma(p00, p11, -pp) - fma(p10, p10, -pp);
       if (!(det > 0.0)) {
         if (threadIdx.x == 0) atomicExch(status, kStatusNumeric);
         det = p00;

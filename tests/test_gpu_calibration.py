@@ -269,3 +269,22 @@ def test_a_ridge_that_outweighs_everything_gives_the_intercept_alone(rate):
     assert (W16 == 0).all() and (W32 == 0).all()
     mean = Y.double().mean(0)
     assert (b.double() - mean).abs().max() <= 2.0 ** -23 * mean.abs().max()       # rounded once to fp32
+
+
+@pytest.mark.parametrize("column", [64, 100, 254, 322])
+def test_a_feature_given_twice_is_reported(column):
+    """Equal features in columns 2 i and 2 i + 1, no ridge term: both pivots of the pair come from the same numbers, so the
+    second is exactly zero whatever the rounding before it, and the fit reports that the matrix is singular."""
+    from paper_2501_19392_b200 import api
+    shape = small_shape(2, 700, 2, oracle.BF16)
+    codec, _ = make(shape)
+    d = shape.d_kv
+    for seed, size in ((1, 1.0), (2, 0.37), (3, 11.0), (4, 1e-3), (5, 1.0), (6, 0.9)):
+        X, X1, Y = (synth.random_16bit((700, d), oracle.BF16, 10 * seed + s, device=DEV) for s in (1, 2, 3))
+        X, X1 = X * size, X1 * size
+        part = X if column < d else X1
+        part[:, column % d + 1] = part[:, column % d]
+        codec.fit_predictor(Y, X, X1 if column >= d else None, rate=0.0)
+        assert codec.poll_status() == api.ERR_NUMERIC, (seed, size)
+    codec.fit_predictor(Y, X, X1, rate=1e-3)
+    assert codec.poll_status() == 0
