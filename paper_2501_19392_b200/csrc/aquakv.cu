@@ -669,7 +669,6 @@ int launch_gram(aquakv_ctx* c, cudaStream_t st, int64_t T, const void* in0, cons
 // ---------------------------------------------------------------------------------------------
 // fused layer kernel (predictor GEMMs + row work in one persistent launch)
 // ---------------------------------------------------------------------------------------------
-constexpr int kLayerRing = 3;       // prediction buffers
 constexpr int kKhatRing = 3;        // waves of reconstructed keys kept when the caller wants none
 
 struct LayerWs {

@@ -38,3 +38,23 @@ def test_layer_calls_equal_the_phases(d, h, T, n, dtype):
     back = codec.decode(ck, sk, cv, sv, Kp, Vp, Wk, Wv, bk, bv)
     assert torch.equal(back[0], kh) and torch.equal(back[1], vh)
     assert codec.poll_status() == 0
+
+
+@pytest.mark.parametrize("d,h,T", [(1024, 1024, 42000), (1024, 64, 30000), (512, 512, 60000), (512, 64, 60000), (256, 256, 90000)])
+def test_repeated_calls_of_many_waves_equal_the_phases(d, h, T):
+    """The prediction ring is reused every three jobs, its lines read and discarded by the row warps, then written by the
+    TMA stores of other CTAs: a store that a late discard or read overtakes would show as wrong rows now and then."""
+    from paper_2501_19392_b200 import api
+    grid = synth.lloyd_grid(16, seed=7, n_samples=1 << 13, iters=8)
+    codec = api.Codec(d, h, h, grid, synth.BF16, synth.hadamard_signs(d, 11), synth.hadamard_signs(d, 12))
+    K, V, Kp, Vp = (synth.random_16bit((T, d), synth.BF16, s, device=DEV) for s in (1, 2, 3, 4))
+    Wk = (synth.random_16bit((d, d), synth.BF16, 5, device=DEV).float() / d ** 0.5).to(K.dtype)
+    Wv = (synth.random_16bit((d, 2 * d), synth.BF16, 6, device=DEV).float() / (2 * d) ** 0.5).to(K.dtype)
+    ck, sk, kh = codec.encode_phase(api.ROLE_KEY, K, Kp, None, Wk)
+    cv, sv, vh = codec.encode_phase(api.ROLE_VALUE, V, Vp, kh, Wv)
+    for _ in range(8):
+        for a, b in zip(codec.encode(K, V, Kp, Vp, Wk, Wv), (ck, sk, cv, sv, kh, vh)):
+            assert torch.equal(a.view(torch.uint8), b.view(torch.uint8))
+        back = codec.decode(ck, sk, cv, sv, Kp, Vp, Wk, Wv)
+        assert torch.equal(back[0], kh) and torch.equal(back[1], vh)
+    assert codec.poll_status() == 0
