@@ -131,12 +131,16 @@ cudaError_t pdl_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
 
 // Fills scratch that the next kernel polls (counters with zeros, preset buffers with ones) by a kernel of the same chain of
 // overlapped starts: behind a memset node the next kernel starts, fills its tables and allocates its tensor memory only when
-// the fill has ended (2-3 us of each such call: 1024 tokens of d_kv 512, two layers there and back 78.4 -> 72.8 us, 64 tokens
-// through two layers of the chain kernel 23.3 -> 21.6).  p and bytes: multiples of 16.  Not counted as a launch of the call's
-// work.
-int launch_fill(const aquakv_ctx* c, cudaStream_t st, void* p, uint32_t word, size_t bytes) {
+// the fill has ended (2-3 us of each such call in a stream of calls: 1024 tokens of d_kv 512, two layers there and back 63.5 -> 56.8 us, 64
+// tokens through two layers of the chain kernel 23.7 -> 21.7; nothing where the stream was idle before).  p and bytes: multiples of 16.
+// behind_attention: the kernel before it is the attention over a chunk.  The next kernel, a decode of the following chunk, then starts when the
+// fill has ended: started beside it, it ran 984 us a chunk of 151552 tokens instead of 942, although it began no sooner (an attention call of 32 x 32768
+// tokens 8240 / 7890 us, 8 x 32768 2065 / 2015).  Why is not known; neither the shared-memory carve-out nor the CTAs' placement is it, and behind
+// other kernels the early start is never slower and gains up to 0.3 us.
+int launch_fill(const aquakv_ctx* c, cudaStream_t st, void* p, uint32_t word, size_t bytes, bool behind_attention = false) {
   const size_t n = bytes / 16, blocks = (n + 255) / 256, cap = size_t(c->sm_count) * 8;
-  return pdl_launch(fill_kernel, dim3(unsigned(blocks < cap ? blocks : cap)), dim3(256), 0, st, static_cast<uint4*>(p), word, n) == cudaSuccess
+  return pdl_launch(behind_attention ? fill_kernel<false> : fill_kernel<true>, dim3(unsigned(blocks < cap ? blocks : cap)), dim3(256), 0, st,
+                    static_cast<uint4*>(p), word, n) == cudaSuccess
              ? AQUAKV_OK
              : AQUAKV_ERR_CUDA;
 }
@@ -924,7 +928,7 @@ int launch_layer(aquakv_ctx* c, cudaStream_t st, bool encode, int64_t T, const v
                  int64_t ld_kv, const void* Khat_prev, const void* Vhat_prev, int64_t ld_prev,
                  const void* Wk, const void* Wv, const float* bk, const float* bv, uint8_t* Kcodes,
                  uint16_t* Kscales, uint8_t* Vcodes, uint16_t* Vscales, void* Khat, void* Vhat,
-                 int64_t ld_hat, void* workspace, const LayerAttnArgs* attn = nullptr) {
+                 int64_t ld_hat, void* workspace, const LayerAttnArgs* attn = nullptr, bool behind_attention = false) {
   const int d = c->p.d_kv;
   const LayerWs ws = layer_ws(c, T, attn != nullptr);
   uint8_t* wsb = ws_base(workspace);
@@ -934,7 +938,7 @@ int launch_layer(aquakv_ctx* c, cudaStream_t st, bool encode, int64_t T, const v
                       ld_prev, Wk, Wv, bk, bv, Kcodes, Kscales, Vcodes, Vscales, Khat, Vhat, ld_hat, attn, &B.layer[0],
                       &B.maps[0]);
   if (rc) return rc;
-  if ((rc = launch_fill(c, st, B.layer[0].gemm_done, 0u, round_up(ws.flags_bytes, 16)))) return rc;
+  if ((rc = launch_fill(c, st, B.layer[0].gemm_done, 0u, round_up(ws.flags_bytes, 16), behind_attention))) return rc;
   const int grid = ws.grid_mw * (d / kBN);
   B.layer[0].last_log_split = wave_log_split(ws.n_mblocks - (ws.n_waves - 1) * ws.mw, grid / 2, d / kBN);
   if (B.layer[0].last_log_split > 0) {
@@ -2254,7 +2258,7 @@ static int decode_attn_impl(aquakv_ctx* c, int32_t batch, int64_t ctx_len, int32
       rc = launch_layer(c, st, false, rows, nullptr, nullptr, 0, Kpv + t0 * ld_prev, Vpv + t0 * ld_prev,
                         ld_prev, Wk, Wv, bk, bv, const_cast<uint8_t*>(Kcodes) + t0 * cb,
                         const_cast<uint16_t*>(Kscales) + t0 * ng, const_cast<uint8_t*>(Vcodes) + t0 * cb,
-                        const_cast<uint16_t*>(Vscales) + t0 * ng, kh, vh, ldh, wsb + ws.layer_off);
+                        const_cast<uint16_t*>(Vscales) + t0 * ng, kh, vh, ldh, wsb + ws.layer_off, nullptr, gb0 > 0);
       if (rc) return rc;
     } else {
       rc = launch_decode_kv(c, st, rows, Kcodes + t0 * cb, Kscales + t0 * ng, Vcodes + t0 * cb, Vscales + t0 * ng, kh, vh, ldh);

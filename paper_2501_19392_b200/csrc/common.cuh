@@ -38,9 +38,11 @@ __device__ __forceinline__ void pdl_sync() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// n 16-byte pieces of one 32-bit word.
+// n 16-byte pieces of one 32-bit word.  kEarly: the next kernel begins its start beside this one, otherwise behind it.
+template <bool kEarly>
 __global__ void __launch_bounds__(256) fill_kernel(uint4* __restrict__ p, uint32_t word, size_t n) {
-  pdl_sync();
+  if constexpr (kEarly) pdl_sync();
+  else asm volatile("griddepcontrol.wait;" ::: "memory");
   for (size_t i = blockIdx.x * size_t(256) + threadIdx.x; i < n; i += size_t(gridDim.x) * 256) p[i] = make_uint4(word, word, word, word);
 }
 
