@@ -638,7 +638,7 @@ def main():
     barrier()
     clocks = sampler.stop()
     ms_total = ev0.elapsed_time(ev1)
-    launches = codec.launch_count() - launches0
+    launches = codec.launch_count() - launches0      # without the fills of scratch
     enc_ms = sum(a.elapsed_time(b) for a, b, _ in mids) / args.steps
     dec_ms = sum(b.elapsed_time(c) for _, b, c in mids) / args.steps
     prof = {name: codec.profile_read(k) for name, k in

@@ -536,13 +536,14 @@ int aquakv_poll_status(aquakv_ctx* ctx, void* cuda_stream);
  */
 int aquakv_selftest_bounded_wait(aquakv_ctx* ctx, int64_t limit_ns, void* cuda_stream);
 
-/* Number of kernels this context has launched since creation (for benchmarks' bookkeeping). */
+/* Number of kernels that do the work of this context's calls, launched since creation (for benchmarks' bookkeeping).  The
+ * small kernel that fills a call's counters or preset buffers before them is not counted, as a memset would not be. */
 int64_t aquakv_launch_count(const aquakv_ctx* ctx);
 
 /*
- * Optional per-kernel timing for benchmarks.  While enabled, every kernel launch of this context
- * is bracketed by a pair of CUDA events on the launching stream (up to 8192 launches; later ones
- * are not recorded).  aquakv_profile_enable(ctx, 1) creates the events on first use (do this
+ * Optional per-kernel timing for benchmarks.  While enabled, every kernel launch that
+ * aquakv_launch_count counts is bracketed by a pair of CUDA events on the launching stream (up to 8192 launches; later
+ * ones are not recorded); fills of scratch lie outside.  aquakv_profile_enable(ctx, 1) creates the events on first use (do this
  * outside stream capture) and clears the record; (ctx, 0) stops recording.
  * aquakv_profile_read waits for the recorded launches of one kernel class and returns their
  * number and summed device time.  Not part of the paper's method: measurement support only.

@@ -132,7 +132,8 @@ cudaError_t pdl_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
 // Fills scratch that the next kernel polls (counters with zeros, preset buffers with ones) by a kernel of the same chain of
 // overlapped starts: behind a memset node the next kernel starts, fills its tables and allocates its tensor memory only when
 // the fill has ended (2-3 us of each such call in a stream of calls: 1024 tokens of d_kv 512, two layers there and back 63.5 -> 56.8 us, 64
-// tokens through two layers of the chain kernel 23.7 -> 21.7; nothing where the stream was idle before).  p and bytes: multiples of 16.
+// tokens through two layers of the chain kernel 23.7 -> 21.7; nothing where the stream was idle before).  p and bytes: multiples of 16.  Neither counted as a launch nor
+// profiled (aquakv_launch_count).
 // behind_attention: the kernel before it is the attention over a chunk.  The next kernel, a decode of the following chunk, then starts when the
 // fill has ended: started beside it, it ran 984 us a chunk of 151552 tokens instead of 942, although it began no sooner (an attention call of 32 x 32768
 // tokens 8240 / 7890 us, 8 x 32768 2065 / 2015).  Why is not known; neither the shared-memory carve-out nor the CTAs' placement is it, and behind
