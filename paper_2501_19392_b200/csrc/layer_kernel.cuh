@@ -17,11 +17,14 @@
 // block for both phases.  Jobs are ordered  K0, K1, V0, K2, V1, ..., so that the value-phase GEMM of
 // a wave (which reads the reconstructed keys of that wave) is issued one job after its key rows.
 //
-// Dependencies (all counted per job j and token-block slot ml, targets NTN):
-//   gemm_done[j][ml]  -- feature tiles of job j written to the ring        (row warps wait; a tile counts kTileWeight, a
-//                        narrow one its part of it)
-//   rows_done[j][ml]  -- CTAs whose row teams have finished job j on token block ml (the value-phase TMA
-//                        producer waits for the key rows of its wave; the GEMM epilogue waits for
+// In the short last wave of a launch of one layer a tile may be 128 or 64 features wide (wave_log_split): more pairs then share a
+// token block, and a pair's slots and feature tile are others than in a full wave.
+//
+// Dependencies (all counted per job j and token-block slot ml):
+//   gemm_done[j][ml]  -- feature tiles of job j written to the ring (row warps wait for kTileWeight * NTN: a whole tile counts
+//                        kTileWeight, a narrow one its part of it)
+//   rows_done[j][ml]  -- CTAs whose row teams have finished job j on token block ml (target: the CTAs that have rows of the block,
+//                        NTN in a full wave; the value-phase TMA producer waits for the key rows of its wave; the GEMM epilogue waits for
 //                        job j - ring size before it overwrites that ring slot)
 // The encoder's last value rows are reported with the key rows of the next job, still before any job that waits for them.
 // Every job waits only on jobs with a smaller index (or the same index of the other role), so the
@@ -70,7 +73,8 @@ constexpr int kWrAttnDecodeWarps = 6;  // beside four attention warps: again 16 
                                        // 2.54 / 2.41 / 2.23 / 2.94 ms per 8 x 32768 tokens)
 static_assert(kWrAttnDecodeWarps <= kWrDecodeWarps, "the decoder's shared memory is sized for kWrDecodeWarps row warps");
 enum RowKind { kRowTeams, kRowWarp, kRowChunks };
-// One warp per row for d_kv <= 512 (rowchunk.cuh), row warps by what their registers hold without spills.  us for 60000 tokens:
+// One warp per row for d_kv <= 512 (rowchunk.cuh), row warps by what their registers hold (without spills but for 16 bytes of the
+// d_kv 256 encoder with blocks shorter than the row).  us for 60000 tokens:
 //   d_kv 512, Hadamard block and group = the row, encoder: teams 292; 10 / 12 / 14 / 16 warps 257 / 279 / 264 / 299;
 //   d_kv 512, encoder with blocks of 64: teams 264, 10 / 14 warps 282 / 286, so the teams stay;
 //   d_kv 512, decoder: teams 184; 10 / 12 / 14 / 16 warps 178 / 175 / 157 / 167 (blocks of 64: 168; 163 / 159 / 147 / 155);
@@ -97,8 +101,14 @@ constexpr int layer_threads() {
   return LayerGeom<kEncode, D, kFull, kAttnHD>::THREADS + (kAttnHD > 0 ? 32 * kAttnWarps : 0);
 }
 
-// The row warps of a CTA may be a few jobs apart, never kJobRing: a job's predictions wait for the rows of three jobs before.
+constexpr int kLayerRing = 3;       // prediction buffers
+static_assert(kLayerRing >= 2, "a job reported with the next one must be out before the job that takes its buffer");
+// Slots of the row warps' hand-offs.  A warp that waits for job g + s while another of its CTA has not finished job g must not meet
+// that job's slot.  The predictions of a job wait for the CTA's rows of kLayerRing jobs before where those lie in the same token
+// block; in a short last wave they lie in another block or nowhere, and the epilogue then looks kLayerRing jobs further back.  With the job of
+// the last wave itself in between s is at most 2 kLayerRing + 1 (played through for 1 to 5 waves and 1 to 4 layers on 8 to 148 CTAs: 5).
 constexpr int kJobRing = 8;
+static_assert(2 * kLayerRing + 1 < kJobRing && (kJobRing & (kJobRing - 1)) == 0, "slots of two jobs would meet");
 
 struct LayerSmemTail {
   uint64_t full[kLayerStagesMax];
@@ -200,9 +210,6 @@ struct LayerArgs {
   int* attn_done;           // [n_waves][mw], zero at launch: attention warps that are done with the block
 };
 
-constexpr int kLayerRing = 3;       // prediction buffers
-static_assert(kLayerRing >= 2, "a job reported with the next one must be out before the job that takes its buffer");
-
 // The layers of one launch.  A launch of several layers (Algorithm 2 / 3 inside Algorithm 4's loop over
 // layers) runs them back to back without a barrier in between: every role walks the layers on its own,
 // the prediction ring and its counters continue across the layer boundary, and a layer's first jobs start
@@ -284,8 +291,10 @@ __device__ __forceinline__ int wave_block_ctas(const WaveRows& w, int block, int
 
 // Longest pause (ns; nanosleep takes up to twice that) between two polls of a counter.  A call of one wave is a chain of
 // four steps, and each waits for the one before, so what a poll comes late is lost (with pauses of 2 us 10 of the 38 us of 1024
-// tokens encoded at d_kv 512); with more waves there is other work in the meantime.  With one poller per CTA, us at pauses of
-// 2048 / 512 / 256: four sequences of 6017 tokens through four layers of a cache policy 836 / 822 / 819, 5000 tokens decoded 62 / 57 / 56.5.
+// tokens encoded at d_kv 512); with more waves there is other work in the meantime.  With one row warp polling per CTA, us at pauses of
+// 2048 / 512 / 256 for every poller: 5000 tokens decoded (two waves) 62 / 57 / 56.5, four sequences of 6017 tokens through four layers of a
+// cache policy (six) 836 / 822 / 819; 2048 / 512: 32768 encoded (eight) 388 / 390, 131072 decoded (29) 895 / 891, 32 x 32768 decoded and
+// attended (33 a chunk) 8420 / 8224.  2048 for the TMA producer and the epilogue alone: 387, 906, 8234.
 __device__ __forceinline__ uint32_t poll_pause(int n_waves) { return n_waves > 1 ? 512u : 128u; }
 
 __device__ __forceinline__ int ld_acquire(const int* p) {
