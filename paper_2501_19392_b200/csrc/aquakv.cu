@@ -1664,7 +1664,7 @@ int aquakv_poll_status(aquakv_ctx* c, void* cuda_stream) {
 
 int aquakv_selftest_bounded_wait(aquakv_ctx* c, int64_t limit_ns, void* cuda_stream) {
   if (c == nullptr || limit_ns <= 0 || limit_ns > int64_t(kWaitLimitNs)) return AQUAKV_ERR_INVALID_ARG;
-  bounded_wait_selftest_kernel<<<1, 32, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
+  bounded_wait_selftest_kernel<<<1, 96, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
       c->d_status, static_cast<unsigned long long>(limit_ns));
   ++c->launches;
   return cudaGetLastError() == cudaSuccess ? AQUAKV_OK : AQUAKV_ERR_CUDA;

@@ -118,21 +118,6 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
   return true;
 }
 
-// One warp waits, with the given limit, on a barrier that nothing ever arrives on: the wait must give
-// up, record the timeout and return.  Used to check the failure path of the bounded waits without
-// disturbing any real kernel (the loop ends on %globaltimer alone).
-__global__ void __launch_bounds__(32) bounded_wait_selftest_kernel(int* status, unsigned long long limit_ns) {
-  __shared__ uint64_t bar;
-  __shared__ int abort_flag;
-  if (threadIdx.x == 0) {
-    mbar_init(&bar, 1);
-    abort_flag = 0;
-    mbar_fence_init();
-  }
-  __syncwarp();
-  if (threadIdx.x == 0) mbar_wait_bounded(&bar, 0u, &abort_flag, status, limit_ns);
-}
-
 // ---------------------------------------------------------------------------------------------
 // TMA (the copies themselves are with the CTA pairs below: bulk tensor copies, never multicast)
 // ---------------------------------------------------------------------------------------------

@@ -303,10 +303,10 @@ __device__ __forceinline__ int ld_acquire(const int* p) {
   return v;
 }
 
-// Spins until *ctr >= target.  Returns false after kWaitLimitNs or if the CTA already aborted.  The pause between two polls
+// Spins until *ctr >= target.  Returns false after limit_ns or if the CTA already aborted.  The pause between two polls
 // doubles up to max_pause: see poll_pause.
 __device__ __forceinline__ bool counter_wait_bounded(const int* ctr, int target, volatile int* abort_flag,
-                                                     int* status, uint32_t max_pause) {
+                                                     int* status, uint32_t max_pause, unsigned long long limit_ns = kWaitLimitNs) {
   if (ld_acquire(ctr) >= target) return true;
   const unsigned long long t0 = global_timer_ns();
   uint32_t spins = 0;
@@ -316,7 +316,7 @@ __device__ __forceinline__ bool counter_wait_bounded(const int* ctr, int target,
     if (pause < max_pause) pause <<= 1;
     if ((++spins & 0x3Fu) == 0) {
       if (*abort_flag) return false;
-      if (global_timer_ns() - t0 > kWaitLimitNs) {
+      if (global_timer_ns() - t0 > limit_ns) {
         *abort_flag = 1;
         atomicExch(status, kStatusTimeout);
         return false;
@@ -335,12 +335,13 @@ __device__ __forceinline__ int ld_acquire_cta(const int* p) {
 // The row warps' wait for the predictions of job `job` (one lane of each team calls it): the first team of the CTA that
 // comes polls the counter in global memory, the others look at shared memory.  (Every team polling for itself: up to 24
 // pollers in each of 148 CTAs held up the very counters that they waited for.)
-__device__ __forceinline__ bool row_wait(LayerSmemTail* tail, int job, const int* ctr, int target, int* status, uint32_t max_pause) {
+__device__ __forceinline__ bool row_wait(LayerSmemTail* tail, int job, const int* ctr, int target, int* status, uint32_t max_pause,
+                                         unsigned long long limit_ns = kWaitLimitNs) {
   const int slot = job & (kJobRing - 1);
   if (ld_acquire_cta(&tail->ready[slot]) >= job) return true;
   volatile int* abort_flag = &tail->abort_flag;
   if (atomicMax(&tail->poller[slot], job) < job) {
-    if (!counter_wait_bounded(ctr, target, abort_flag, status, max_pause)) return false;
+    if (!counter_wait_bounded(ctr, target, abort_flag, status, max_pause, limit_ns)) return false;
     asm volatile("st.release.cta.shared::cta.s32 [%0], %1;" ::"r"(smem_u32(&tail->ready[slot])), "r"(job) : "memory");
     return true;
   }
@@ -350,7 +351,7 @@ __device__ __forceinline__ bool row_wait(LayerSmemTail* tail, int job, const int
     __nanosleep(64);
     if ((++spins & 0xFu) == 0) {
       if (*abort_flag) return false;
-      if (global_timer_ns() - t0 > 2 * kWaitLimitNs) {       // the polling warp has given up before
+      if (global_timer_ns() - t0 > 2 * limit_ns) {           // the polling warp has given up before
         *abort_flag = 1;
         atomicExch(status, kStatusTimeout);
         return false;
@@ -358,6 +359,39 @@ __device__ __forceinline__ bool row_wait(LayerSmemTail* tail, int job, const int
     }
   }
   return true;
+}
+
+// The failure paths of the three kinds of wait, one warp each, every one for something that never comes: a barrier that nothing
+// arrives on, a counter that nothing raises, and (a row warp behind another that polls) a word in shared memory that
+// nobody writes.  Each must give up after its limit, raise its abort flag and say so; only then *status reads kStatusTimeout.
+// The loops end on %globaltimer alone.
+__global__ void __launch_bounds__(96) bounded_wait_selftest_kernel(int* status, unsigned long long limit_ns) {
+  __shared__ uint64_t bar;
+  __shared__ LayerSmemTail tail[2];          // of the poller and of the warp behind one
+  __shared__ int bar_abort, told[3], gave_up[3];
+  const int warp = threadIdx.x >> 5;
+  if (threadIdx.x == 0) {
+    mbar_init(&bar, 1);
+    mbar_fence_init();
+    bar_abort = 0;
+    for (int i = 0; i < 2; ++i) {
+      tail[i].abort_flag = 0;
+      for (int k = 0; k < kJobRing; ++k) tail[i].poller[k] = tail[i].ready[k] = 0;
+    }
+    tail[1].poller[1] = 1;
+    for (int i = 0; i < 3; ++i) told[i] = gave_up[i] = 0;
+  }
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) {
+    if (warp == 0) gave_up[0] = !mbar_wait_bounded(&bar, 0u, &bar_abort, &told[0], limit_ns);
+    else gave_up[warp] = !row_wait(&tail[warp - 1], 1, status, 1, &told[warp], 512u, limit_ns);      // a status word is never above 0
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    bool all = bar_abort != 0 && tail[0].abort_flag != 0 && tail[1].abort_flag != 0;
+    for (int i = 0; i < 3; ++i) all = all && gave_up[i] && told[i] == kStatusTimeout;
+    if (all) atomicExch(status, kStatusTimeout);
+  }
 }
 
 // A row team's report on job `job`; true for the last of the CTA's `teams`, which reports for all of them (its fence then
