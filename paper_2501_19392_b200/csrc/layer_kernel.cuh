@@ -258,8 +258,8 @@ __device__ __forceinline__ int layer_key_job(int wave) { return wave == 0 ? 0 : 
 __device__ __forceinline__ int layer_value_job(int wave, int n_waves) {
   return wave == n_waves - 1 ? 2 * n_waves - 1 : 2 * wave + 2;
 }
-// A value job that is followed by the key rows of a full wave (in which every CTA has rows).
-__device__ __forceinline__ bool later_report(int j, int n_waves) { return j >= 2 && (j & 1) == 0 && j + 1 < 2 * n_waves - 3; }
+// Value job j is followed by the key rows of a full wave, in which every CTA has rows.
+__device__ __forceinline__ bool later_report(int j, int n_jobs) { return j >= 2 && j < n_jobs - 4; }
 
 // Row work of a wave is spread evenly over ALL CTAs: CTA slot s takes rows [s*rpc, (s+1)*rpc) of
 // the wave, rpc = the power of two >= rows / CTAs.  For a full wave this is rpc = 128 / NTN rows of
@@ -893,18 +893,20 @@ layer_kernel(const __grid_constant__ LayerBatch<kBatch> B) {
         // stores.  The decoder leaves those discards out; the encoder reports such rows with the key rows of the
         // next job, whose release covers them (later_report), and else releases where the slot is taken again.
         // Measured against reports without a release and discards all the same (which was a race), us: 32768 tokens of d_kv 1024
-        // encoded 392 / 388, 60000 694 / 696, of d_kv 512 277 / 279; 131072 of d_kv 1024 decoded 907 / 892, 60000 of d_kv 512 181 / 179.
-        // A release of its own for every report costs 1 to 2 %, encoded rows without discards 1.5 to 2 %, decoded rows reported later 4 to 5 %.
+        // encoded 387 / 386, 60000 684 / 685, 200000 2200 / 2245, 60000 of d_kv 512 272 / 275; 131072 of d_kv 1024 decoded 890 / 881, 60000 of d_kv 512
+        // 177 / 175.  A release of its own for every report costs 1 to 2 %, encoded rows without discards 1 to 1.5 % from 30000 tokens on (but 60000 and
+        // fewer gain by the later report), decoded rows reported later 4 to 5 %; a fourth buffer would halve what the long encodes lose, but
+        // the decoder loses by it and the workspace grows.
         if (ph == 0 || l + 1 < n_layers) {
           fence_acq_rel_gpu();
           fence_proxy_async_all();
-          if (kEncode && ph == 0 && l + 1 == n_layers && j > 0 && later_report(j - 1, a.n_waves))
-            atomicAdd(a.rows_done + (j - 1) * a.mw + ml, 1);
+          if (kEncode && ph == 0 && l + 1 == n_layers && later_report(j - 1, n_jobs))
+            atomicAdd(a.rows_done + (j - 1) * a.mw + rb, 1);       // both are full waves: the same token block
           atomicAdd(a.rows_done + j * a.mw + rb, 1);
         } else if (kAttnHD > 0) {
           fence_acq_rel_gpu();
           atomicAdd(a.rows_done + j * a.mw + rb, 1);
-        } else if (!(kEncode && later_report(j, a.n_waves))) {
+        } else if (!(kEncode && later_report(j, n_jobs))) {
           if (kEncode && j + kLayerRing < n_jobs) {
             fence_acq_rel_gpu();
             fence_proxy_async_all();
