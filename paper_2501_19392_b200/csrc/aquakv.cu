@@ -134,13 +134,14 @@ cudaError_t pdl_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
 // the fill has ended (2-3 us of each such call in a stream of calls: 1024 tokens of d_kv 512, two layers there and back 63.5 -> 56.8 us, 64
 // tokens through two layers of the chain kernel 23.7 -> 21.7; nothing where the stream was idle before).  p and bytes: multiples of 16.  Neither counted as a launch nor
 // profiled (aquakv_launch_count).
-// behind_attention: the kernel before it is the attention over a chunk.  The next kernel, a decode of the following chunk, then starts when the
-// fill has ended: started beside it, it ran 984 us a chunk of 151552 tokens instead of 942, although it began no sooner (an attention call of 32 x 32768
-// tokens 8240 / 7890 us, 8 x 32768 2065 / 2015).  Why is not known; neither the shared-memory carve-out nor the CTAs' placement is it, and behind
-// other kernels the early start is never slower and gains up to 0.3 us.
-int launch_fill(const aquakv_ctx* c, cudaStream_t st, void* p, uint32_t word, size_t bytes, bool behind_attention = false) {
+// late: the next kernel starts when the fill has ended instead of beside it, for two long decodes that run slower started beside it although
+// they begin no sooner: that of a chunk behind the attention over the chunk before (984 us instead of 942 for 151552 tokens; 32 x 32768 tokens
+// attended 8240 / 7890, 8 x 32768 2065 / 2015), and that of several layers (eight layers of 9300 tokens 586 / 560, 20000 1106 / 1057, 32768 1790 / 1737).
+// Why is not known; neither the shared-memory carve-out nor the CTAs' placement is it.  Other calls gain up to 0.9 us by the early start (5000
+// tokens decoded 53.9 / 54.6, 20000 of d_kv 512 encoded 99.1 / 100.1), eight layers encoded up to half a percent.
+int launch_fill(const aquakv_ctx* c, cudaStream_t st, void* p, uint32_t word, size_t bytes, bool late = false) {
   const size_t n = bytes / 16, blocks = (n + 255) / 256, cap = size_t(c->sm_count) * 8;
-  return pdl_launch(behind_attention ? fill_kernel<false> : fill_kernel<true>, dim3(unsigned(blocks < cap ? blocks : cap)), dim3(256), 0, st,
+  return pdl_launch(late ? fill_kernel<false> : fill_kernel<true>, dim3(unsigned(blocks < cap ? blocks : cap)), dim3(256), 0, st,
                     static_cast<uint4*>(p), word, n) == cudaSuccess
              ? AQUAKV_OK
              : AQUAKV_ERR_CUDA;
@@ -929,7 +930,7 @@ int launch_layer(aquakv_ctx* c, cudaStream_t st, bool encode, int64_t T, const v
                  int64_t ld_kv, const void* Khat_prev, const void* Vhat_prev, int64_t ld_prev,
                  const void* Wk, const void* Wv, const float* bk, const float* bv, uint8_t* Kcodes,
                  uint16_t* Kscales, uint8_t* Vcodes, uint16_t* Vscales, void* Khat, void* Vhat,
-                 int64_t ld_hat, void* workspace, const LayerAttnArgs* attn = nullptr, bool behind_attention = false) {
+                 int64_t ld_hat, void* workspace, const LayerAttnArgs* attn = nullptr, bool late_fill = false) {
   const int d = c->p.d_kv;
   const LayerWs ws = layer_ws(c, T, attn != nullptr);
   uint8_t* wsb = ws_base(workspace);
@@ -939,7 +940,7 @@ int launch_layer(aquakv_ctx* c, cudaStream_t st, bool encode, int64_t T, const v
                       ld_prev, Wk, Wv, bk, bv, Kcodes, Kscales, Vcodes, Vscales, Khat, Vhat, ld_hat, attn, &B.layer[0],
                       &B.maps[0]);
   if (rc) return rc;
-  if ((rc = launch_fill(c, st, B.layer[0].gemm_done, 0u, round_up(ws.flags_bytes, 16), behind_attention))) return rc;
+  if ((rc = launch_fill(c, st, B.layer[0].gemm_done, 0u, round_up(ws.flags_bytes, 16), late_fill))) return rc;
   const int grid = ws.grid_mw * (d / kBN);
   B.layer[0].last_log_split = wave_log_split(ws.n_mblocks - (ws.n_waves - 1) * ws.mw, grid / 2, d / kBN);
   if (B.layer[0].last_log_split > 0) {
@@ -1133,7 +1134,7 @@ int run_layers(aquakv_ctx* c, bool encode, int64_t T, int32_t L, const void* con
                       Khat[li], Vhat[li], ld_hat, nullptr, &B.layer[i], &B.maps[i]);
       if (rc) return rc;
     }
-    if ((rc = launch_fill(c, st, wsb + ws.flags_off, 0u, size_t(n) * ws.flags_stride))) return rc;
+    if ((rc = launch_fill(c, st, wsb + ws.flags_off, 0u, size_t(n) * ws.flags_stride, !encode))) return rc;
     {
       ProfScope prof(c, st, AQUAKV_KERNEL_LAYER);
       if (encode) {
