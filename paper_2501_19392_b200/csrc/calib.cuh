@@ -311,8 +311,8 @@ __global__ void fit_prepare_kernel(const float* __restrict__ P, int slices, int 
 // What bounds it: the chain diagonal tile -> tile below it -> next diagonal tile, n / 64 times; the arithmetic
 // (n^3 / 3 + n^2 d) would take 0.2 ms of the 2048-feature fit.  A step of the chain, by time stamps: flag and tiles 1.8 us, last
 // product 2.4, diagonal tile 10, store and flag 1.1, its tile to the one below 1.3, triangular solve 1.6, store and flag 0.7.
-// d = 1024, n = 1024 and 2048 together: forward 0.92 ms (stamps), back 0.44 (what is left of the call's gain) (with one pivot at a time and solves of a column at a time
-// 1.40 and 0.58; a launch per step of 32 columns 8.4).
+// d = 1024, n = 1024 and 2048: forward 0.29 and 0.59 ms, back 0.12 and 0.29 (ncu, serialised; with one pivot at a time and solves of a column
+// at a time both fits took 1.36 forward and 0.57 back; with a launch per step of 32 columns 8.4 in all).
 // ---------------------------------------------------------------------------------------------
 constexpr int kFitThreads = 256;
 constexpr int kFitTile = kFitNB * kFitLd;                                  // doubles of a tile in shared memory
