@@ -129,3 +129,31 @@ def test_strided_rows_and_calls_without_reconstructions(d, h, T):
     assert codec.poll_status() == 0
     for i, o in enumerate(out):
         assert torch.equal(o[:, :d], want[4 + i % 2]) and (o[:, d:] == 3.0).all()
+
+
+@pytest.mark.parametrize("T", [14000, 18432, 23100])
+def test_several_layers_of_many_waves_in_one_launch_equal_layer_by_layer(T):
+    """Four to six waves: the last layer reports its value rows with the next key rows, the layers before it by themselves."""
+    from paper_2501_19392_b200 import chain
+    d, L = 1024, 3
+    codec = make_codec(d, d, 16)
+    row = lambda s: synth.random_16bit((T, d), synth.BF16, s, device=DEV)
+    K, V = [row(10 + l) for l in range(L)], [row(20 + l) for l in range(L)]
+    W = lambda n, s: (synth.random_16bit((d, n), synth.BF16, s, device=DEV).float() / n ** 0.5).bfloat16()
+    Wk, Wv = [None] + [W(d, 30 + l) for l in range(1, L)], [None] + [W(2 * d, 40 + l) for l in range(1, L)]
+    ref, hats = chain.CompressedCache.empty(codec, L, T, DEV), []
+    for l in range(L):
+        prev = hats[-1] if l else (None, None)
+        hats.append(codec.encode(K[l], V[l], *prev, Wk[l], Wv[l], None, None, ref.Kcodes[l], ref.Kscales[l], ref.Vcodes[l], ref.Vscales[l])[4:])
+    for _ in range(3):
+        got = chain.CompressedCache.empty(codec, L, T, DEV)
+        Kh, Vh = ([torch.empty_like(K[0]) for _ in range(L)] for _ in range(2))
+        codec.encode_chain(K, V, Wk, Wv, got.Kcodes, got.Kscales, got.Vcodes, got.Vscales, Khat=Kh, Vhat=Vh)
+        Kb, Vb = ([torch.empty_like(K[0]) for _ in range(L)] for _ in range(2))
+        codec.decode_chain(ref.Kcodes, ref.Kscales, ref.Vcodes, ref.Vscales, Wk, Wv, Khat=Kb, Vhat=Vb)
+        assert codec.poll_status() == 0
+        for l in range(L):
+            for a, b in ((got.Kcodes, ref.Kcodes), (got.Kscales, ref.Kscales), (got.Vcodes, ref.Vcodes), (got.Vscales, ref.Vscales)):
+                assert torch.equal(a[l], b[l]), l
+            for a, b in ((Kh[l], hats[l][0]), (Vh[l], hats[l][1]), (Kb[l], hats[l][0]), (Vb[l], hats[l][1])):
+                assert torch.equal(a, b), l
